@@ -28,7 +28,7 @@ int tc_gemm_error(cudaStream_t s);
 int tc_set_wait_cycles(long long cycles);
 
 // FP64-accurate GEMM from exact BF16 products of digit slices (tc_gemm.cu).
-// ozaki_split: S slices of the rows of X (rows x K, FP64) into `out`
+// ozaki_split: S slices of the rows of X (rows x K, FP64), [K/8][S][rows][8], into `out`
 // (ozaki_slice_bytes), *e = per-row exponents inside `out`.
 size_t ozaki_slice_bytes(int rows, int K, int S);
 int ozaki_split(cudaStream_t s, const double* X, int rows, int K, int S, void* out, int** e);

@@ -39,24 +39,47 @@ static __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t byt
                  : "memory");
 }
 
-// Bounded wait for the completion of the phase with the given parity.
+static __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Bounded wait for the completion of the phase with the given parity.  A
+// phase that is complete already costs one try: the clock and the limit (in
+// global memory) are read only by a wait that has to go on.
 static __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
     const long long lim = g_tc_wait_cycles;
     while (true) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
+        if (mbar_try(bar, parity)) return true;
         if (clock64() - t0 > lim) {
             atomicExch(&g_tc_error, 1);
             return false;
         }
     }
+}
+
+// The same wait by a whole converged warp, with a warp-uniform result (so the
+// code after it stays uniform: the tensor-core instructions take their
+// descriptors from uniform registers).
+static __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+
+// One lane of a converged warp.
+static __device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile(
+        "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(e));
+    return e != 0;
 }
 
 static __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
