@@ -13,7 +13,7 @@ OUT = os.path.join(HERE, '_build')
 LIB = os.path.join(OUT, 'librte.so')
 ARCH = ['-gencode', 'arch=compute_103a,code=sm_103a']
 SOURCES = ['setup_host.cpp', 'mg_host.cpp', 'server.cpp', 'kernels.cu', 'mg.cu', 'tc_gemm.cu',
-           'rte.cu', 'dgemm_static.cu', 'tune.cpp', 'e0_direct.cu', 'ec_direct.cu', 'h2.cu',
+           'rte.cu', 'dgemm_static.cu', 'tune.cpp', 'e0_direct.cu', 'ec_direct.cu', 'ec_kron.cu', 'h2.cu',
            'h2_build.cpp']
 # host files whose floating point must round the same on every host (no
 # contraction into fused multiply-adds)

@@ -19,6 +19,7 @@
 
 #include "device.h"
 #include "mg.h"
+#include "mg_device.cuh"
 #include "persist.cuh"
 #include "rte_internal.h"
 
@@ -26,48 +27,7 @@ namespace rte {
 
 namespace {
 
-constexpr float kOmega = 0.7f;          // Jacobi damping
 constexpr int kCoarseSweeps = 30;       // coarsest-level sweeps without a dense inverse
-
-__device__ __forceinline__ int nbr(int i, int dir, int m, int n) {
-    const int off[7] = {0, 1, -1, m + 1, -(m + 1), m + 2, -(m + 2)};
-    const int j = i + off[dir];
-    return j < 0 ? 0 : (j >= n ? n - 1 : j);
-}
-
-// restriction P^T: fine node q of coarse node I's list (the fine nodes that
-// interpolate from I, with their weights; width Cv.rwid, zero-weight padding)
-__device__ __forceinline__ int restrict_src(const MGDeviceLevel& Cv, int I, int q, float& w) {
-    const size_t k = (size_t)I * Cv.rwid + q;
-    w = __ldg(Cv.rw + k);
-    return __ldg(Cv.ridx + k);
-}
-
-// prolongation: coarse nodes (and weights) interpolating fine node i; the
-// coarse mesh is the floor(mf/2)-mesh, and for odd mf the last fine column
-// and row take the values of the ones before them
-__device__ __forceinline__ void prolong_src(int i, int mf, int& c0, int& c1, float& w0,
-                                            float& w1) {
-    const int mc = mf / 2;
-    const int x = min(i % (mf + 1), 2 * mc), y = min(i / (mf + 1), 2 * mc);
-    if (!(x & 1) && !(y & 1)) {
-        c0 = c1 = (y / 2) * (mc + 1) + x / 2;
-        w0 = 1.f;
-        w1 = 0.f;
-    } else if ((x & 1) && !(y & 1)) {
-        c0 = (y / 2) * (mc + 1) + (x - 1) / 2;
-        c1 = c0 + 1;
-        w0 = w1 = 0.5f;
-    } else if (!(x & 1)) {
-        c0 = ((y - 1) / 2) * (mc + 1) + x / 2;
-        c1 = c0 + (mc + 1);
-        w0 = w1 = 0.5f;
-    } else {
-        c0 = ((y - 1) / 2) * (mc + 1) + (x - 1) / 2;
-        c1 = c0 + (mc + 2);
-        w0 = w1 = 0.5f;
-    }
-}
 
 // Grid-stride loop over the items (i, c) = (e / nc, e % nc) of an n x nc
 // array, with the quotient and remainder advanced incrementally (no division
@@ -1084,7 +1044,8 @@ struct EcMG {
     int L, nrhs, d, nu, G;
     int Q;                 // Kronecker terms of the levels (0: explicit blocks)
     bool dense;
-    const float* cinv;     // [(n_c d)][(n_c d)]
+    const float* cinv;     // [n_c d][cld]
+    int cld;               // its row stride: n_c d rounded up to 4
     const float* Gq;       // angular blocks of the terms [Q][d][d] (Q > 0)
     const MGDeviceLevel* lev;   // [L], in device memory
 };
@@ -1298,7 +1259,7 @@ __device__ bool ec_vcycle(const EcMG& mg, const float* sG, GridBar* bar, float*&
             for (unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw;
                  w += (gridDim.x * blockDim.x) >> 5) {
                 const int r = (int)(w / (unsigned)N), q = (int)(w % (unsigned)N);
-                const float* row = mg.cinv + (size_t)q * N;
+                const float* row = mg.cinv + (size_t)q * mg.cld;
                 const float* b = Lv.B + (size_t)r * N;
                 // 6 independent load pairs in flight per lane and trip
                 constexpr int U = 6;
@@ -1792,9 +1753,8 @@ int e0_cg_lo(cudaStream_t s, const DevSystem& d, const double* B, double* X, int
 
 size_t coarse_cg_work_bytes(const DevSystem& d, int nrhs) {
     const size_t n = (size_t)nrhs * d.nRp * d.dP;
-    return 3 * (((n * 8) + 255) / 256 * 256) + (((n * 4) + 255) / 256 * 256) +
-           ((9 * (size_t)nrhs * 8 + 255) / 256 * 256) + (((size_t)nrhs * 8 + 255) / 256 * 256) +
-           256;
+    return 4 * (((n * 8) + 255) / 256 * 256) + ((9 * (size_t)nrhs * 8 + 255) / 256 * 256) +
+           (((size_t)nrhs * 8 + 255) / 256 * 256) + 256;
 }
 
 int coarse_cg(cudaStream_t s, const DevSystem& d, const double* B, double* X, int nrhs,
@@ -1804,6 +1764,9 @@ int coarse_cg(cudaStream_t s, const DevSystem& d, const double* B, double* X, in
     if (work_bytes < coarse_cg_work_bytes(d, nrhs))
         return fail(RTE_ERR_ARG, "coarse CG workspace too small");
     if (nrhs > d.ecmg.cap_cols) return fail(RTE_ERR_ARG, "coarse multigrid sized for fewer RHS");
+    if (ec_kron_takes(d, nrhs))
+        return ec_kron_cg(s, d, B, X, nrhs, tol, maxit, work, status_dev, f32_products,
+                          g_wait_limit_ns, g_trace_buf, g_trace_cap);
     const size_t n = (size_t)nrhs * d.nRp * d.dP;
     char* p = static_cast<char*>(work);
     EcArgs a;
@@ -1833,6 +1796,7 @@ int coarse_cg(cudaStream_t s, const DevSystem& d, const double* B, double* X, in
     a.ldf = ec_direct_ld(d.m, d.dP);
     a.mg = view<EcMG>(d.ecmg);
     a.mg.nrhs = nrhs;
+    a.mg.cld = d.ecmg.cld;
     a.mg.d = d.dP;
     a.mg.G = d.dP <= 8 ? 8 : (d.dP <= 16 ? 16 : 32);
     a.mg.Q = d.ecmg.Q;

@@ -19,6 +19,9 @@ struct MGDeviceLevel {
     const float* val = nullptr;    // E_c: [7][n][d][d], blocks transposed
     const float* dinv = nullptr;   // E_c: [n][d][d] inverse diagonal blocks, transposed
     const float* sv = nullptr;     // E_0: six spatial parts [n][7][8]; E_c: Q terms [n][7][Qp]
+    // E_c in Kronecker form: which terms a node has (bit c: sigma class c,
+    // bit 7: the boundary terms)
+    const unsigned char* kmask = nullptr;
     float *X = nullptr, *Xt = nullptr, *B = nullptr;   // work vectors
     // restriction from the next finer level: for each node of this level,
     // rwid fine nodes and weights (zero-weight padding); unset on level 0
@@ -31,6 +34,7 @@ struct MGDevice {
     int L = 0, nu = 2, cap_cols = 0;
     bool dense = false;
     const float* cinv = nullptr;   // coarsest dense inverse(s)
+    int cld = 0;                   // E_c only: row stride of cinv (a multiple of 4)
     int Q = 0;                     // E_c only: number of Kronecker terms (0: blocks)
     const float* G = nullptr;      // E_c only: angular blocks of the terms [Q][d][d]
     const float* w8 = nullptr;     // E_0 only: per-direction weights [nSp][8], six used

@@ -480,6 +480,13 @@ int upload_mg_kron(rte_handle* h, const MGHost& mh, int cols, int d, int Q,
                 for (int q = 0; q < Q; ++q)
                     sk[((size_t)i * 7 + dir) * Qp + q] = (float)ell[((size_t)q * 7 + dir) * D.n + i];
         RTE_TRY(upload(h, &D.sv, sk));
+        std::vector<unsigned char> mask(D.n, 0);
+        for (int i = 0; i < D.n; ++i)
+            for (int dir = 0; dir < 7; ++dir)
+                for (int q = 2; q < Q; ++q)
+                    if (ell[((size_t)q * 7 + dir) * D.n + i] != 0.0)
+                        mask[i] |= q < 4 ? 0x80 : 1 << (q - 4) / 4;
+        RTE_TRY(upload(h, &D.kmask, mask));
         std::vector<float> di((size_t)D.n * dd);
         std::vector<double> blk(dd), inv(dd);
         for (int i = 0; i < D.n; ++i) {
@@ -539,6 +546,23 @@ int upload_mg(rte_handle* h, const MGHost& mh, int cols, int bs, bool block_dinv
         RTE_TRY(dalloc(h, &D.B, nv));
     }
     return RTE_OK;
+}
+
+// Inverse of the coarsest E_c (N x N) with its rows padded by zeros to a
+// multiple of 4 (16-byte loads).
+int upload_coarse_inverse(rte_handle* h, int N, const std::vector<double>& A, MGDevice& out) {
+    std::vector<float> inv;
+    RTE_TRY(spd_inverse_batch(h, N, 1, A, inv));
+    const size_t ld = ((size_t)N + 3) & ~(size_t)3;
+    if (ld != (size_t)N) {
+        std::vector<float> pad((size_t)N * ld, 0.f);
+        for (int r = 0; r < N; ++r)
+            std::copy(inv.begin() + (size_t)r * N, inv.begin() + (size_t)(r + 1) * N,
+                      pad.begin() + r * ld);
+        inv.swap(pad);
+    }
+    out.cld = (int)ld;
+    return upload(h, &out.cinv, inv);
 }
 
 // The multigrid of E_c uses its Kronecker form when it has at most this many
@@ -722,9 +746,7 @@ int setup_multigrid(rte_handle* h, const HostSystem& hs, SetupClock* clk) {
                                     A[(size_t)(i * dP + a) * N + j * dP + b] += sq * g[a * dP + b];
                         }
                     }
-                std::vector<float> inv;
-                RTE_TRY(spd_inverse_batch(h, N, 1, A, inv));
-                RTE_TRY(upload(h, &d.ecmg.cinv, inv));
+                RTE_TRY(upload_coarse_inverse(h, N, A, d.ecmg));
             }
         } else {
             RTE_TRY(build_hierarchy(hs.m, hs.st, h->h_ec, 1, dP, kDenseCoarseNodes, mh));
@@ -732,10 +754,8 @@ int setup_multigrid(rte_handle* h, const HostSystem& hs, SetupClock* clk) {
             if (d.ecmg.dense) {
                 std::vector<double> A;
                 coarse_dense_matrix(mh.levels.back(), {}, 1, dP, A);
-                std::vector<float> inv;
                 const int N = (mh.levels.back().m + 1) * (mh.levels.back().m + 1) * dP;
-                RTE_TRY(spd_inverse_batch(h, N, 1, A, inv));
-                RTE_TRY(upload(h, &d.ecmg.cinv, inv));
+                RTE_TRY(upload_coarse_inverse(h, N, A, d.ecmg));
             }
         }
         // FP64 level-0 blocks of the CG's own apply
