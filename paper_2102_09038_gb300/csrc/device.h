@@ -81,7 +81,7 @@ struct DevSystem {
     // E_0 level-0 stencil coefficients per direction, ELL [7][nRp][nSp]
     const double* e0coef;
     // direct route of E_0^{-1}: inverses of the row Schur complements of every
-    // direction block, [nSp][m+1][ld][ld] (e0_direct.cu); one of the two set
+    // direction block, [nSp][m+1] records (e0_direct.cu); one of the two set
     bool e0_direct = false;
     const float* e0lu32 = nullptr;
     const double* e0lu64 = nullptr;

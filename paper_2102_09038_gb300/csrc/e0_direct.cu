@@ -8,19 +8,33 @@
 // block of size b = m + 1:
 //   A_yy      tridiagonal (self, +x, -x),
 //   A_y,y-1   two diagonals (-y: node (x, y-1), -x-y: node (x-1, y-1)),
-//   A_y,y+1 = A_y+1,y^T.
-// Its block LDU factorisation A = L D U has D = diag(S_y) with the Schur
-// complements S_0 = A_00, S_y = A_yy - A_y,y-1 S_y-1^{-1} A_y-1,y, and is
-// stored as the explicit inverses S_y^{-1} (dense, symmetric, b x b).  The
-// solve is then a forward and a backward sweep over the rows, each a dense
-// matrix-vector product with S_y^{-1} plus the two-diagonal couplings:
-//   forward   w_y = S_y^{-1} (b_y - A_y,y-1 w_y-1)
-//   backward  x_y = w_y - S_y^{-1} (A_y,y+1 x_y+1)
-// so the solve streams the factor from HBM twice, in wide coalesced loads,
-// with one block per direction (and all right-hand sides of the direction
-// in that block, so the factor is read once for up to kRB of them).
+//   A_y,y+1 = A_y+1,y^T   (+y: node (x, y+1), +x+y: node (x+1, y+1)).
+// The rows are eliminated from both ends towards the middle row h = b / 2:
+// S_0 = A_00, S_y = A_yy - A_y,y-1 S_y-1^{-1} A_y-1,y for y < h, the same from
+// the last row upwards for y > h, and S_h with both corrections.  Kept are
+// the explicit inverses S_y^{-1} (dense, symmetric, b x b).  The solve runs
+// both chains at once, each by one block of a two-block cluster:
+//   towards h   w_y = S_y^{-1} (b_y - A_y,y' w_y')       y' the row before
+//   at h        x_h = S_h^{-1} (b_h - A_h,h-1 w_h-1 - A_h,h+1 w_h+1)
+//               (each block, after exchanging the two w)
+//   back        x_y = w_y - S_y^{-1} (A_y,y' x_y')       y' the row after
+// so a direction takes b dependent steps of two blocks instead of 2 b - 1 of
+// one.
 //
-// Setup factorises in FP64 (one block per direction, S_y in shared memory,
+// What bounds it: reading the factor, twice, from HBM on large meshes; on
+// small ones the chain of steps, each a wait for its record, a few products
+// and three block barriers.  Hence each S_y^{-1} is kept by the tiles of its
+// upper triangle (8 x 8, the diagonal ones full: 0.59 of the dense rows at
+// b = 129), in one record with its row's coupling coefficients, so a step is
+// one bulk copy into a ring of shared-memory slots; as many blocks share an
+// SM as the slots allow, and where a chain's right-hand side fits in shared
+// memory (small meshes) the steps touch no global memory but the copies and
+// the stores of x.  Measured, us per solve (one right-hand side): 128 x 128 /
+// 256 directions FP32 1075 -> 640, FP64 10580 -> 5000;
+// 32 x 32 / 64 directions FP32 137 -> 37, FP64 325 -> 66; 96 x 96 / 1024
+// directions FP32 2480 -> 1230.
+//
+// Setup factorises in FP64 (two blocks per direction, S_y in shared memory,
 // Gauss-Jordan inversion); the factor is kept in FP64 (FP64 mode) or FP32
 // (mixed modes, where E_0^{-1} is a preconditioner under the FP64 outer
 // residual).
@@ -35,14 +49,15 @@ namespace rte {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kRB = 4;   // right-hand sides per sweep of the factor
-// largest mesh of the route: the FP32 solve stages two factor blocks of
-// ld x ld floats (ld <= 160) in shared memory beside its vectors
+constexpr int kThreads = 256;        // of the factorisation
+constexpr int kRB = 4;               // right-hand sides per sweep of the factor
+constexpr int kMaxParts = 6;         // groups that share a tile row, at most
+// largest mesh of the route: the set-up holds one b x b FP64 matrix in
+// shared memory
 constexpr int kMaxM = 156;
-constexpr int kE = 3;    // elements of a [kRB][ld] array per thread (ld <= 160)
+constexpr int kSmemPerSm = 226 * 1024;
 
-// Limit of one wait for a factor block (SM clock cycles; ~2 s at 2 GHz),
+// Limit of one wait for a factor record (SM clock cycles; ~2 s at 2 GHz),
 // and the flag a wait that ran out sets.
 __device__ long long g_e0_wait_cycles = 4000000000ll;
 __device__ int g_e0_error = 0;
@@ -52,41 +67,78 @@ __device__ __forceinline__ double cf(const double* coef, int nRp, int nSp, int d
     return coef[((size_t)dir * nRp + node) * nSp + k];
 }
 
-// Factorisation of direction block k = blockIdx.x.  G: FP64 scratch of b x b
-// per direction (S_y-1^{-1} while S_y is formed); out32 / out64: the inverses,
-// [k][y][ld][ld], zero-padded to ld.
-__global__ void __launch_bounds__(kThreads) k_e0_factor(int m, int nSp, int ld,
+// Threads of the solve's products for one and for up to kRB right-hand sides,
+// at most (one more warp copies): with four blocks on an SM 48 and 64
+// registers each.
+__host__ __device__ constexpr int e0_threads(int NR) { return NR == 1 ? 288 : 224; }
+
+// A row's record, in elements: [A pair | tiles | B pair] with nt = ceil(b / 8)
+// tile rows and bp = 8 nt; the A pair holds the coefficients towards row y - 1
+// (-y at x, then bp later -x-y at x), the B pair those towards y + 1 (+y, then
+// +x+y); pairs are padded to whole tiles.
+__host__ __device__ __forceinline__ int e0_nt(int m) { return (m + 8) / 8; }
+__host__ __device__ __forceinline__ int e0_tiles(int nt) { return nt * (nt + 1) / 2; }
+__host__ __device__ __forceinline__ int e0_pair(int nt) { return (16 * nt + 63) / 64 * 64; }
+__host__ __device__ __forceinline__ int e0_record(int nt) { return 64 * e0_tiles(nt) + 2 * e0_pair(nt); }
+// tile (I, J), I <= J, and element (r, c) of tile t: rows permuted by the
+// tile and 16-byte pieces by the row, so that eight lanes reading one row
+// each (16 bytes) and four times eight lanes reading one row of neighbouring
+// tiles (one element each) both meet distinct banks
+__host__ __device__ __forceinline__ int e0_tile(int nt, int I, int J) {
+    return I * nt - I * (I - 1) / 2 + J - I;
+}
+template <typename T>
+__host__ __device__ __forceinline__ int e0_elem(int t, int r, int c) {
+    constexpr int CH = 16 / sizeof(T), NCH = 8 / CH;   // elements per piece, pieces per row
+    return 64 * t + ((r ^ (t & 3)) * 8) + (((c / CH) ^ (r / (8 / NCH))) * CH) + c % CH;
+}
+
+// One chain (or the middle row) of direction block k = blockIdx.x: part 0 the
+// rows 0 .. h-1 downwards, 1 the rows b-1 .. h+1 upwards, 2 the row h.  G:
+// FP64 scratch of two b x b per direction (the last inverse of either chain);
+// out32 / out64: the records [k][y].
+__global__ void __launch_bounds__(kThreads) k_e0_factor(int m, int nSp, int middle,
                                                         const double* __restrict__ coef,
                                                         double* __restrict__ G,
                                                         float* __restrict__ out32,
                                                         double* __restrict__ out64) {
     extern __shared__ double sm[];
-    const int b = m + 1, nRp = b * b, k = blockIdx.x;
+    const int b = m + 1, nRp = b * b, k = blockIdx.x, h = b / 2;
+    const int part = middle ? 2 : (int)blockIdx.y;
+    const int nt = e0_nt(m), bp = 8 * nt, rec = e0_record(nt);
     double* S = sm;                 // b x b, row-major, leading dimension b
     double* colp = S + b * b;       // column p before elimination
     double* rowp = colp + b;        // row p after scaling
-    double* Gk = G + (size_t)k * b * b;
     const int bb = b * b;
-    for (int y = 0; y < b; ++y) {
-        // S_y = A_yy - A_y,y-1 S_y-1^{-1} A_y-1,y
+    double* Gk = G + (size_t)k * 2 * bb;
+    const int rows = part == 0 ? h : part == 1 ? b - 1 - h : 1;
+    for (int n = 0; n < rows; ++n) {
+        const int y = part == 0 ? n : part == 1 ? b - 1 - n : h;
+        // S_y = A_yy - sum over the rows y' eliminated before it (y - 1 and /
+        // or y + 1) of A_y,y' S_y'^{-1} A_y',y
         for (int e = threadIdx.x; e < bb; e += blockDim.x) {
             const int r = e / b, c = e - r * b;
-            const int nr = y * b + r;
+            const int nr = y * b + r, nc = y * b + c;
             double v = 0.0;
             if (r == c) v = cf(coef, nRp, nSp, 0, nr, k);
             else if (c == r + 1) v = cf(coef, nRp, nSp, 1, nr, k);
             else if (c == r - 1) v = cf(coef, nRp, nSp, 2, nr, k);
-            if (y > 0) {
-                const int nc = y * b + c;
-                const double lr0 = cf(coef, nRp, nSp, 4, nr, k);   // (r, y-1)
-                const double lr1 = r > 0 ? cf(coef, nRp, nSp, 6, nr, k) : 0.0;   // (r-1, y-1)
-                const double lc0 = cf(coef, nRp, nSp, 4, nc, k);
-                const double lc1 = c > 0 ? cf(coef, nRp, nSp, 6, nc, k) : 0.0;
-                double s = lr0 * lc0 * Gk[r * b + c];
-                if (c > 0) s += lr0 * lc1 * Gk[r * b + c - 1];
-                if (r > 0) s += lr1 * lc0 * Gk[(r - 1) * b + c];
-                if (r > 0 && c > 0) s += lr1 * lc1 * Gk[(r - 1) * b + c - 1];
-                v -= s;
+            for (int side = 0; side < 2; ++side) {
+                const bool from = side == 0 ? (part != 1 && y > 0)
+                                            : (part != 0 && y < b - 1);
+                if (!from) continue;
+                const double* Gs = Gk + (size_t)side * bb;
+                const int d0 = side == 0 ? 4 : 3, d1 = side == 0 ? 6 : 5, s = side == 0 ? -1 : 1;
+                const bool hr = r + s >= 0 && r + s < b, hc = c + s >= 0 && c + s < b;
+                const double lr0 = cf(coef, nRp, nSp, d0, nr, k);
+                const double lr1 = hr ? cf(coef, nRp, nSp, d1, nr, k) : 0.0;
+                const double lc0 = cf(coef, nRp, nSp, d0, nc, k);
+                const double lc1 = hc ? cf(coef, nRp, nSp, d1, nc, k) : 0.0;
+                double a = lr0 * lc0 * Gs[r * b + c];
+                if (hc) a += lr0 * lc1 * Gs[r * b + c + s];
+                if (hr) a += lr1 * lc0 * Gs[(r + s) * b + c];
+                if (hr && hc) a += lr1 * lc1 * Gs[(r + s) * b + c + s];
+                v -= a;
             }
             S[e] = v;
         }
@@ -115,412 +167,482 @@ __global__ void __launch_bounds__(kThreads) k_e0_factor(int m, int nSp, int ld,
             }
             __syncthreads();
         }
-        // symmetrised inverse to the factor and to the scratch of the next row
-        const size_t o = ((size_t)k * b + y) * ld * ld;
-        for (int e = threadIdx.x; e < ld * ld; e += blockDim.x) {
-            const int r = e / ld, c = e - r * ld;
-            const double v = (r < b && c < b) ? 0.5 * (S[r * b + c] + S[c * b + r]) : 0.0;
-            if (out32) out32[o + e] = (float)v;
-            if (out64) out64[o + e] = v;
-            if (r < b && c < b) Gk[r * b + c] = v;
+        // symmetrised inverse and couplings to the record, and the inverse
+        // to the scratch of the next row
+        const size_t o = ((size_t)k * b + y) * rec;
+        auto put = [&](int at, double v) {
+            if (out32) out32[o + at] = (float)v;
+            if (out64) out64[o + at] = v;
+        };
+        for (int e = threadIdx.x; e < bp * bp; e += blockDim.x) {
+            const int r = e / bp, c = e - r * bp, I = r >> 3, J = c >> 3;
+            const bool in = r < b && c < b;
+            const double v = in ? 0.5 * (S[r * b + c] + S[c * b + r]) : 0.0;
+            if (in && part < 2) Gk[(size_t)part * bb + r * b + c] = v;
+            if (I > J) continue;
+            const int t = e0_tile(nt, I, J);
+            put(e0_pair(nt) + (out32 ? e0_elem<float>(t, r & 7, c & 7) : e0_elem<double>(t, r & 7, c & 7)), v);
+        }
+        const int pw = e0_pair(nt);
+        for (int e = threadIdx.x; e < 2 * pw; e += blockDim.x) {
+            const int up = e / pw, f = e - up * pw, q = f / bp, x = f - q * bp;
+            const int dir = up ? (q ? 5 : 3) : (q ? 6 : 4);
+            put(up ? rec - pw + f : f, q < 2 && x < b ? cf(coef, nRp, nSp, dir, y * b + x, k) : 0.0);
         }
         __syncthreads();
     }
 }
 
-// four consecutive factor entries, streamed (each is read once per sweep)
-__device__ __forceinline__ void ld4s(const double* p, double (&o)[4]) {
-    const double2 a = __ldcs(reinterpret_cast<const double2*>(p));
-    const double2 c = __ldcs(reinterpret_cast<const double2*>(p) + 1);
-    o[0] = a.x; o[1] = a.y; o[2] = c.x; o[3] = c.y;
-}
-
-// out[r][x] = sum_c Sinv[c][x] v[r][c] for the nr right-hand sides of the
-// sweep (Sinv symmetric: row c read as column c, four consecutive x per
-// load).  Thread t takes the four rows 4 (t % nq4) .. + 3 and the column chunk
-// t / nq4 of ng; partial sums meet in red.
-template <typename T>
-__device__ __forceinline__ void matvec(const T* __restrict__ Sinv, int b, int ld, int nr,
-                                       const T* v, T* red, T* out) {
-    const int nq4 = ld >> 2;
-    const int ng = max(1, min(b, (int)blockDim.x / nq4));
-    const int cw = (b + ng - 1) / ng;
-    const int q = threadIdx.x % nq4, g = threadIdx.x / nq4;
-    if (g < ng) {
-        T acc[kRB][4];
-#pragma unroll
-        for (int r = 0; r < kRB; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = T(0);
-        const int c0 = g * cw, c1 = min(b, c0 + cw);
-#pragma unroll 4
-        for (int c = c0; c < c1; ++c) {
-            T s[4];
-            ld4s(Sinv + (size_t)c * ld + 4 * q, s);
-#pragma unroll
-            for (int r = 0; r < kRB; ++r) {
-                if (r < nr) {
-                    const T vc = v[r * ld + c];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) acc[r][u] = fma(s[u], vc, acc[r][u]);
-                }
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < kRB; ++r)
-            if (r < nr)
-#pragma unroll
-                for (int u = 0; u < 4; ++u) red[((size_t)g * kRB + r) * ld + 4 * q + u] = acc[r][u];
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nr * b; e += blockDim.x) {
-        const int r = e / b, x = e - r * b;
-        T s = T(0);
-        for (int gg = 0; gg < ng; ++gg) s += red[((size_t)gg * kRB + r) * ld + x];
-        out[r * ld + x] = s;
-    }
-    __syncthreads();
-}
-
-// X = E_0^{-1} B for direction k = blockIdx.x, every right-hand side, in
-// sweeps of kRB right-hand sides.  X holds w_y after the forward sweep.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_e0_direct(int m, int nSp, int nrhs, int ld,
-                                                        const T* __restrict__ fac,
-                                                        const double* __restrict__ coef,
-                                                        const double* __restrict__ B,
-                                                        double* __restrict__ X) {
-    extern __shared__ __align__(128) unsigned char smraw[];
-    T* sm = reinterpret_cast<T*>(smraw);
-    const int b = m + 1, nRp = b * b, k = blockIdx.x;
-    T* v = sm;                    // [kRB][ld] right-hand side of the product
-    T* prev = v + kRB * ld;       // [kRB][ld] w_y-1 (forward) or x_y+1 (backward)
-    T* res = prev + kRB * ld;     // [kRB][ld] the product
-    T* red = res + kRB * ld;      // [ng][kRB][ld] partial sums
-    const T* fk = fac + (size_t)k * b * ld * ld;
-    for (int r0 = 0; r0 < nrhs; r0 += kRB) {
-        const int nr = min(kRB, nrhs - r0);
-        // forward: w_y = S_y^{-1} (b_y - A_y,y-1 w_y-1)
-        for (int y = 0; y < b; ++y) {
-            for (int e = threadIdx.x; e < kRB * ld; e += blockDim.x) {
-                const int r = e / ld, x = e - r * ld;
-                T val = T(0);
-                if (r < nr && x < b) {
-                    const int node = y * b + x;
-                    val = (T)B[((size_t)(r0 + r) * nRp + node) * nSp + k];
-                    if (y > 0) {
-                        val -= (T)cf(coef, nRp, nSp, 4, node, k) * prev[r * ld + x];
-                        if (x > 0) val -= (T)cf(coef, nRp, nSp, 6, node, k) * prev[r * ld + x - 1];
-                    }
-                }
-                v[e] = val;
-            }
-            __syncthreads();
-            matvec<T>(fk + (size_t)y * ld * ld, b, ld, nr, v, red, res);
-            for (int e = threadIdx.x; e < kRB * ld; e += blockDim.x) {
-                const int r = e / ld, x = e - r * ld;
-                prev[e] = res[e];
-                if (r < nr && x < b)
-                    X[((size_t)(r0 + r) * nRp + y * b + x) * nSp + k] = (double)res[e];
-            }
-            __syncthreads();
-        }
-        // backward: x_m = w_m (held in prev); x_y = w_y - S_y^{-1} (A_y,y+1 x_y+1)
-        for (int y = b - 2; y >= 0; --y) {
-            for (int e = threadIdx.x; e < kRB * ld; e += blockDim.x) {
-                const int r = e / ld, x = e - r * ld;
-                T val = T(0);
-                if (r < nr && x < b) {
-                    const int node = y * b + x;
-                    val = (T)cf(coef, nRp, nSp, 3, node, k) * prev[r * ld + x];
-                    if (x + 1 < b) val += (T)cf(coef, nRp, nSp, 5, node, k) * prev[r * ld + x + 1];
-                }
-                v[e] = val;
-            }
-            __syncthreads();
-            matvec<T>(fk + (size_t)y * ld * ld, b, ld, nr, v, red, res);
-            for (int e = threadIdx.x; e < kRB * ld; e += blockDim.x) {
-                const int r = e / ld, x = e - r * ld;
-                T xv = T(0);
-                if (r < nr && x < b) {
-                    double* p = X + ((size_t)(r0 + r) * nRp + y * b + x) * nSp + k;
-                    xv = (T)(*p) - res[e];
-                    *p = (double)xv;
-                }
-                prev[e] = xv;
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// ------------------------------------------------------------------------
-// FP32 solve with the factor staged in shared memory by TMA bulk copies (one
-// copy per half block, each into its own slot, so copies overlap the
-// products).  The blocks are used in the order y = 0..m (forward) then
-// m-1..0 (backward): step t takes block t < b ? t : 2b - 2 - t.  The
-// right-hand side, the coupling coefficients and (backward) the forward
-// result of the next step are loaded into registers one step ahead.
-
 __device__ __forceinline__ uint32_t sh_addr(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// Bounded wait for the phase of parity `par` of the mbarrier at `bar`.
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t par) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(par)
+        : "memory");
+    return ok != 0;
+}
+
+// Bounded wait for the phase of parity `par` of the mbarrier at `bar`.  The
+// limit (in global memory) is read only by a wait that has gone on for a
+// while: its latency would otherwise be part of every wait that does not
+// succeed at once.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t par) {
-    const long long t0 = clock64(), lim = g_e0_wait_cycles;
+    if (mbar_try(bar, par)) return true;
+    const long long t0 = clock64();
     while (true) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(bar), "r"(par)
-            : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > lim) {
+        for (int i = 0; i < 64; ++i)
+            if (mbar_try(bar, par)) return true;
+        if (clock64() - t0 > g_e0_wait_cycles) {
             atomicExch(&g_e0_error, 1);
             return false;
         }
     }
 }
 
-// Thread 0: one bulk copy of `bytes` (a multiple of 16, both addresses
+// One thread: one bulk copy of `bytes` (a multiple of 16, both addresses
 // 16-byte aligned) from global src into shared dst, completing on bar.
-__device__ __forceinline__ void tma_block(void* dst, const void* src, uint32_t bytes,
+__device__ __forceinline__ void tma_block(uint32_t dst, const void* src, uint32_t bytes,
                                           uint32_t bar) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
                  : "memory");
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-        ::"r"(sh_addr(dst)), "l"(src), "r"(bytes), "r"(bar)
+        ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
         : "memory");
 }
 
-// The block's product in two halves of its rows c (the columns of the
-// product, S being symmetric): half h covers c in [h hb, min(b, (h + 1) hb)),
-// hb = ceil(b / 2), contiguous in memory.  Each half goes through its own
-// shared-memory slot, so the copy of one half of the next block runs while
-// the other half is used, and a block needs about half the shared memory of
-// a whole one: two blocks of threads fit on an SM.
-__device__ __forceinline__ void matvec_half(const float* __restrict__ S, int c_lo, int c_hi,
-                                            int ld, int nr, int q, int g, int cw,
-                                            const float* v, float (&acc)[kRB][4]) {
-    const int c0 = max(c_lo, g * cw), c1 = min(c_hi, (g + 1) * cw);
-#pragma unroll 4
-    for (int c = c0; c < c1; ++c) {
-        const float4 sv = *reinterpret_cast<const float4*>(S + (size_t)(c - c_lo) * ld + 4 * q);
+// all threads of both blocks of the cluster; earlier writes to the peer's
+// shared memory are visible after it
+__device__ __forceinline__ void cluster_meet() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// loads by shared-memory address: one element, or a 16-byte piece
+__device__ __forceinline__ void lds(uint32_t p, float& v) {
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(p));
+}
+__device__ __forceinline__ void lds(uint32_t p, double& v) {
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(p));
+}
+__device__ __forceinline__ void lds16(uint32_t p, float* v) {
+    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "r"(p));
+}
+__device__ __forceinline__ void lds16(uint32_t p, double* v) {
+    asm volatile("ld.shared.v2.f64 {%0,%1}, [%2];" : "=d"(v[0]), "=d"(v[1]) : "r"(p));
+}
+
+__device__ __forceinline__ void sts(uint32_t p, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(p), "f"(v) : "memory");
+}
+__device__ __forceinline__ void sts(uint32_t p, double v) {
+    asm volatile("st.shared.f64 [%0], %1;" ::"r"(p), "d"(v) : "memory");
+}
+template <typename T>
+__device__ __forceinline__ T ldv(uint32_t p) {
+    T v;
+    lds(p, v);
+    return v;
+}
+
+// acc[r] += s . v[r] over the eight values at shared address p + r stride, in
+// two short chains (they round less than one over the whole row)
+template <typename T, int NR>
+__device__ __forceinline__ void e0_dot(const T (&s)[8], uint32_t p, uint32_t stride, T (&acc)[NR]) {
+    constexpr int CH = 16 / sizeof(T);
 #pragma unroll
-        for (int r = 0; r < kRB; ++r)
-            if (r < nr) {
-                const float vc = v[r * ld + c];
-                acc[r][0] = fmaf(sv.x, vc, acc[r][0]);
-                acc[r][1] = fmaf(sv.y, vc, acc[r][1]);
-                acc[r][2] = fmaf(sv.z, vc, acc[r][2]);
-                acc[r][3] = fmaf(sv.w, vc, acc[r][3]);
-            }
+    for (int r = 0; r < NR; ++r) {
+        T u[8];
+#pragma unroll
+        for (int i = 0; i < 8 / CH; ++i) lds16(p + r * stride + 16 * i, u + CH * i);
+        T a = s[0] * u[0], c4 = s[4] * u[4];
+#pragma unroll
+        for (int c = 1; c < 4; ++c) {
+            a = fma(s[c], u[c], a);
+            c4 = fma(s[4 + c], u[4 + c], c4);
+        }
+        acc[r] += a + c4;
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_e0_direct_tma(int m, int nSp, int nrhs, int ld,
-                                                               const float* __restrict__ fac,
-                                                               const double* __restrict__ coef,
-                                                               const double* __restrict__ B,
-                                                               double* __restrict__ X) {
+// X = E_0^{-1} B for direction k = blockIdx.x / 2, every right-hand side, in
+// sweeps of up to kRB; block side 0 of the cluster takes the rows from 0, side
+// 1 those from b - 1, both the middle row.  Eight lanes own eight consecutive
+// rows of the product (one each) and read their tiles by rows right of the
+// diagonal, by columns left of it; P groups of eight share a tile row and meet
+// in `part`.  HIST: the chain's right-hand side, and then its w, stay in
+// shared memory; else they are read one step ahead and w waits in X.
+template <typename T, bool HIST, int NR>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(e0_threads(NR) + 32, sizeof(T) == 4 ? 4 : 2)
+k_e0_solve(int m, int nSp, int nrhs, int P, int slots, const T* __restrict__ fac,
+           const double* __restrict__ B, double* __restrict__ X) {
     extern __shared__ __align__(128) unsigned char smraw[];
-    const int b = m + 1, nRp = b * b, k = blockIdx.x;
-    const int hb = (b + 1) / 2;                     // rows of the first half
-    const size_t blk = (size_t)ld * ld, slot_elems = (size_t)hb * ld;
-    float* slot = reinterpret_cast<float*>(smraw);  // [2][hb][ld]
-    float* v = slot + 2 * slot_elems;               // [kRB][ld]
-    float* prev = v + kRB * ld;                     // [kRB][ld]
-    float* res = prev + kRB * ld;                   // [kRB][ld]
-    float* red = res + kRB * ld;                    // [ng][kRB][ld]
-    __shared__ __align__(8) unsigned long long bars[2];
-    const uint32_t bar[2] = {sh_addr(&bars[0]), sh_addr(&bars[1])};
-    const float* fk = fac + (size_t)k * b * blk;
-    const int steps = 2 * b - 1;
-    auto block_of = [&](int t) { return t < b ? t : 2 * b - 2 - t; };
-    // half h of the block of step t: source and byte count
-    auto half_src = [&](int t, int h) { return fk + (size_t)block_of(t) * blk + (size_t)h * slot_elems; };
-    auto half_bytes = [&](int h) {
-        return (uint32_t)((size_t)(h == 0 ? hb : b - hb) * ld * sizeof(float));
-    };
-    const int nq4 = ld >> 2;
-    const int ng = max(1, min(b, (int)blockDim.x / nq4));
-    const int cw = (b + ng - 1) / ng;
-    const int q = threadIdx.x % nq4, g = threadIdx.x / nq4;
-    if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar[0]) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar[1]) : "memory");
+    constexpr int SZ = sizeof(T), CH = 16 / SZ, NCH = 8 / CH, RB = 8 * SZ, kE = NR;
+    const int b = m + 1, nRp = b * b, h = b / 2, nt = e0_nt(m), bp = 8 * nt, rec = e0_record(nt);
+    const int k = blockIdx.x >> 1, side = blockIdx.x & 1, tid = threadIdx.x;
+    const int n = side == 0 ? h : b - 1 - h;   // rows of the chain
+    const int passes = (nrhs + NR - 1) / NR;
+    const int nthr = (int)blockDim.x - 32;     // of the products; the last warp copies
+    __shared__ __align__(8) unsigned long long bars[16];   // full and empty, per slot
+    const uint32_t full0 = sh_addr(bars), empty0 = full0 + 64;
+    // Byte addresses in shared memory: the ring (tiles on their own size:
+    // their elements' addresses are formed by XOR), the product's right-hand
+    // side, the row before, the other chain's last w (twice), the partial
+    // products, and with HIST the chain's rows.
+    const uint32_t recb = rec * SZ, pairb = e0_pair(nt) * SZ, rowb = (uint32_t)bp * SZ, vecb = NR * rowb;
+    const uint32_t ring = (sh_addr(smraw) + 511) & ~511u, aV = ring + slots * recb, aPrev = aV + vecb,
+                   aMid = aPrev + vecb, aPart = aMid + 2 * vecb, aHist = aPart + P * vecb;
+    const T* fk = fac + (size_t)k * b * rec;
+    if (tid == 0) {
+        for (int s = 0; s < slots; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(full0 + 8 * s) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(empty0 + 8 * s), "r"(nthr / 32)
+                         : "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    unsigned uses = 0;   // completed phases of each slot's barrier (equal for both)
-    for (int r0 = 0; r0 < nrhs; r0 += kRB) {
-        const int nr = min(kRB, nrhs - r0);
-        if (threadIdx.x == 0) {
-            // the previous sweep's reads of both slots are done (its last
-            // barrier); order them before the copies' writes
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            tma_block(slot, half_src(0, 0), half_bytes(0), bar[0]);
-            if (b > hb) tma_block(slot + slot_elems, half_src(0, 1), half_bytes(1), bar[1]);
+    cluster_meet();   // the peer runs: its shared memory may be written
+    if (tid >= nthr) {
+        // The last warp keeps the ring full, one record per step and without
+        // the pair of coefficients the step does not use.  It has nothing to
+        // exchange at the middle row: it arrives there ahead (its copies must
+        // go on while the products wait for each other) and waits when the
+        // sweep's copies are issued.
+        int slot = 0, done = 0;
+        uint32_t ph = 1;   // a fresh barrier passes a wait for the phase before
+        bool ok = true;
+        for (int pass = 0; pass < passes; ++pass) {
+            asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+            if (tid == nthr)
+                for (int t = 0; t <= 2 * n && ok; ++t) {
+                    if (!mbar_wait(empty0 + 8 * slot, ph)) { ok = false; break; }
+                    // every read of the slot came before its arrivals: order
+                    // them before the copy
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    const int j = t < n ? t : 2 * n - t;   // chain row, n: the middle
+                    const int y = j == n ? h : side == 0 ? j : b - 1 - j;
+                    const bool needA = t == n || (t < n) == (side == 0), needB = t == n || !needA;
+                    const uint32_t o0 = needA ? 0 : pairb, o1 = needB ? recb : recb - pairb;
+                    tma_block(ring + slot * recb + o0,
+                              reinterpret_cast<const char*>(fk + (size_t)y * rec) + o0, o1 - o0,
+                              full0 + 8 * slot);
+                    ++done;
+                    if (++slot == slots) { slot = 0; ph ^= 1; }
+                }
+            __syncwarp();
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         }
-        // registers for step t: B (forward) or the forward result w (backward),
-        // and the two coupling coefficients of the row
-        double pb[kE], pc0[kE], pc1[kE];
-        auto fetch = [&](int t) {
-            const bool fw = t < b;
-            const int y = block_of(t);
+        // after a timeout: the copies still in flight land before the block
+        // leaves
+        if (tid == nthr && !ok)
+            for (int q = max(0, done - slots); q < done; ++q)
+                mbar_wait(full0 + 8 * (q % slots), (uint32_t)(q / slots) & 1u);
+        return;
+    }
+    // barrier of the products' threads alone
+    auto block_sync = [&]() { asm volatile("barrier.sync 1, %0;" ::"r"(nthr) : "memory"); };
+    const int g = tid >> 3, lane = tid & 7, I = g % nt, p = g / nt;
+    const bool work = p < P;
+    const int J0 = p * nt / P, J1 = (p + 1) * nt / P;
+    // this group's tiles: columns of (J0 .. Jc - 1, I), rows of (I, Jr .. J1 - 1)
+    const int Jc = min(J1, I), Jr = max(J0, I), colt = e0_tile(nt, J0, I), rowt = e0_tile(nt, I, Jr);
+    const uint32_t aOut = aPart + p * vecb + (8 * I + lane) * SZ;
+    // the coefficient pairs towards the row before (forward) and after, and
+    // the neighbour in x they reach besides the node itself
+    const uint32_t pairA = 0, pairB = recb - pairb;
+    const uint32_t fpair = side == 0 ? pairA : pairB, bpair = side == 0 ? pairB : pairA;
+    const int fs = side == 0 ? -1 : 1;
+    bool ok = true;   // this thread's waits; after one that ran out the steps
+                      // go on without stores, so that the cluster meets
+    int slot = 0;
+    uint32_t ph = 0;
+    for (int pass = 0; pass < passes; ++pass) {
+        const int r0 = pass * NR, nr = min(NR, nrhs - r0);
+        // this thread's elements of a row: one x, and the right-hand sides
+        // rfirst, rfirst + rstep, ...; byte offsets of x and of the neighbours
+        // in x the two pairs reach (the node itself where there is none: the
+        // coefficient is zero there)
+        const int rfirst = NR == 1 ? 0 : tid / bp, x = tid - rfirst * bp;
+        const int rstep = NR == 1 ? 1 : nthr / bp;
+        const bool mine_x = NR == 1 ? tid < bp : rfirst < rstep;
+        const uint32_t xb = x * SZ;
+        const int nbf = (x + fs >= 0 && x + fs < b) ? fs * SZ : 0;
+        const int nbb = (x - fs >= 0 && x - fs < b) ? -fs * SZ : 0;
+        bool own[kE], in[kE];
+        uint32_t eb[kE];
+#pragma unroll
+        for (int j = 0; j < kE; ++j) {
+            const int r = rfirst + j * rstep;
+            // (a last sweep of fewer carries zeros for the others)
+            own[j] = mine_x && r < NR;
+            in[j] = own[j] && x < b && r < nr;
+            eb[j] = r * rowb + xb;
+        }
+        const size_t at0 = ((size_t)(r0 + rfirst) * nRp + x) * nSp + k,
+                     atr = (size_t)rstep * nRp * nSp;
+        auto at = [&](int j) { return at0 + j * atr; };   // place in B and X, without the row
+        const size_t ystep = (size_t)b * nSp;
+        auto chain_at = [&](int j) { return (size_t)(side == 0 ? j : b - 1 - j) * ystep; };
+        // read ahead: the next step's b towards the middle, w on the way back
+        T nxt[kE];
+        auto ahead = [&](const double* src, size_t row) {
+#pragma unroll
+            for (int j = 0; j < kE; ++j) nxt[j] = in[j] ? (T)src[at(j) + row] : T(0);
+        };
+        ahead(B, HIST || n == 0 ? h * ystep : chain_at(0));
+        if constexpr (HIST) {
+            for (int c = 0; c < n; ++c)
+#pragma unroll
+                for (int j = 0; j < kE; ++j)
+                    if (own[j])
+                        sts(aHist + c * vecb + eb[j], in[j] ? (T)B[at(j) + chain_at(c)] : T(0));
+        }
+        // the record of the next step
+        auto record = [&]() -> uint32_t {
+            if (ok && !mbar_wait(full0 + 8 * slot, ph)) ok = false;
+            return ring + slot * recb;
+        };
+        auto pair = [&](uint32_t c, uint32_t u, int j, int nb) {
+            T a = ldv<T>(c + xb) * ldv<T>(u + eb[j]);
+            return a + ldv<T>(c + rowb + xb) * ldv<T>(u + eb[j] + nb);
+        };
+        // sum[j] = element j of S^{-1} v for the record at R, whose slot is
+        // then given back
+        auto product = [&](uint32_t R, T (&sum)[kE]) {
+            block_sync();   // v is complete
+            if (work) {
+                T acc[NR], s[8];
+#pragma unroll
+                for (int r = 0; r < NR; ++r) acc[r] = T(0);
+                const uint32_t tiles = R + pairb;
+                int tl = colt;
+#pragma unroll 2
+                for (int J = J0; J < Jc; ++J) {
+                    const uint32_t q = tiles + tl * 8 * RB + ((tl & 3) * RB) + lane * SZ;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        lds(q ^ (uint32_t)(c * RB | (c / (8 / NCH)) << 4), s[c]);
+                    e0_dot<T, NR>(s, aV + J * RB, rowb, acc);
+                    tl += nt - J - 1;
+                }
+                tl = rowt;
+#pragma unroll 2
+                for (int J = Jr; J < J1; ++J, ++tl) {
+                    const uint32_t q = tiles + tl * 8 * RB + ((lane ^ (tl & 3)) * RB) + ((lane / (8 / NCH)) << 4);
+#pragma unroll
+                    for (int i = 0; i < NCH; ++i) lds16(q ^ (uint32_t)(i << 4), s + CH * i);
+                    e0_dot<T, NR>(s, aV + J * RB, rowb, acc);
+                }
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    sts(aOut + r * rowb, acc[r]);
+            }
+            // the slot is free once every warp has read it
+            __syncwarp();
+            if ((tid & 31) == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty0 + 8 * slot) : "memory");
+            if (++slot == slots) { slot = 0; ph ^= 1; }
+            block_sync();   // the partial products are complete
 #pragma unroll
             for (int j = 0; j < kE; ++j) {
-                const int e = threadIdx.x + j * kThreads;
-                const int r = e / ld, x = e - r * ld;
-                pb[j] = pc0[j] = pc1[j] = 0.0;
-                if (e < kRB * ld && r < nr && x < b) {
-                    const int node = y * b + x;
-                    if (fw) {
-                        pb[j] = B[((size_t)(r0 + r) * nRp + node) * nSp + k];
-                        if (y > 0) {
-                            pc0[j] = cf(coef, nRp, nSp, 4, node, k);
-                            if (x > 0) pc1[j] = cf(coef, nRp, nSp, 6, node, k);
-                        }
-                    } else {
-                        pb[j] = X[((size_t)(r0 + r) * nRp + node) * nSp + k];
-                        pc0[j] = cf(coef, nRp, nSp, 3, node, k);
-                        if (x + 1 < b) pc1[j] = cf(coef, nRp, nSp, 5, node, k);
-                    }
-                }
+                if (!own[j]) continue;
+                T q[kMaxParts];
+#pragma unroll
+                for (int u = 0; u < kMaxParts; ++u)
+                    q[u] = u < P ? ldv<T>(aPart + u * vecb + eb[j]) : T(0);
+                sum[j] = ((q[0] + q[1]) + (q[2] + q[3])) + (q[4] + q[5]);
             }
         };
-        fetch(0);
-        for (int t = 0; t < steps; ++t) {
-            const bool fw = t < b;
-            const int y = block_of(t);
-            // the product's right-hand side from the registers and prev
+        // towards the middle: w_y
+        T sum[kE];
+        for (int t = 0; t < n; ++t) {
+            const uint32_t R = record();
 #pragma unroll
             for (int j = 0; j < kE; ++j) {
-                const int e = threadIdx.x + j * kThreads;
-                if (e >= kRB * ld) continue;
-                const int r = e / ld, x = e - r * ld;
-                float val = 0.f;
-                if (r < nr && x < b) {
-                    if (fw) {
-                        val = (float)pb[j];
-                        if (y > 0) {
-                            val -= (float)pc0[j] * prev[r * ld + x];
-                            if (x > 0) val -= (float)pc1[j] * prev[r * ld + x - 1];
-                        }
-                    } else {
-                        val = (float)pc0[j] * prev[r * ld + x];
-                        if (x + 1 < b) val += (float)pc1[j] * prev[r * ld + x + 1];
-                    }
+                if (!own[j]) continue;
+                T v = T(0);
+                if (in[j]) {
+                    v = HIST ? ldv<T>(aHist + t * vecb + eb[j]) : nxt[j];
+                    if (t > 0) v -= pair(R + fpair, aPrev, j, nbf);
                 }
-                v[e] = val;
+                sts(aV + eb[j], v);
             }
-            // the backward epilogue needs this step's w: keep it before the
-            // registers move on to the next step
-            float wv[kE];
-#pragma unroll
-            for (int j = 0; j < kE; ++j) wv[j] = (float)pb[j];
-            if (t + 1 < steps) fetch(t + 1);
-            __syncthreads();
-            float acc[kRB][4];
-#pragma unroll
-            for (int r = 0; r < kRB; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
-            for (int h = 0; h < 2; ++h) {
-                const int c_lo = h * hb, c_hi = h == 0 ? hb : b;
-                if (c_hi <= c_lo) continue;
-                const bool ok = mbar_wait(bar[h], uses & 1u);
-                if (__syncthreads_or(!ok)) {
-                    // a copy did not arrive in time: let the other slot's copy
-                    // finish (bounded) and leave; the host reads g_e0_error
-                    if (threadIdx.x == 0 && h == 0 && b > hb) mbar_wait(bar[1], uses & 1u);
-                    return;
-                }
-                if (g < ng) matvec_half(slot + h * slot_elems, c_lo, c_hi, ld, nr, q, g, cw, v, acc);
-                __syncthreads();
-                if (threadIdx.x == 0 && t + 1 < steps) {
-                    // every thread's reads of this slot are done (barrier above)
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    tma_block(slot + h * slot_elems, half_src(t + 1, h), half_bytes(h), bar[h]);
-                }
-            }
-            ++uses;
-            if (g < ng)
-#pragma unroll
-                for (int r = 0; r < kRB; ++r)
-                    if (r < nr)
-                        *reinterpret_cast<float4*>(red + ((size_t)g * kRB + r) * ld + 4 * q) =
-                            make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
-            __syncthreads();
-            for (int e = threadIdx.x; e < nr * ld; e += blockDim.x) {
-                float sum = 0.f;
-                const int r = e / ld, x = e - r * ld;
-                for (int gg = 0; gg < ng; ++gg) sum += red[((size_t)gg * kRB + r) * ld + x];
-                res[r * ld + x] = sum;
-            }
-            __syncthreads();
+            if constexpr (!HIST) ahead(B, t + 1 < n ? chain_at(t + 1) : h * ystep);
+            product(R, sum);
 #pragma unroll
             for (int j = 0; j < kE; ++j) {
-                const int e = threadIdx.x + j * kThreads;
-                if (e >= kRB * ld) continue;
-                const int r = e / ld, x = e - r * ld;
-                float out = 0.f;
-                if (r < nr && x < b) {
-                    out = fw ? res[e] : wv[j] - res[e];
-                    X[((size_t)(r0 + r) * nRp + y * b + x) * nSp + k] = (double)out;
-                }
-                prev[e] = out;
+                if (!own[j]) continue;
+                sts(aPrev + eb[j], sum[j]);
+                if constexpr (HIST) sts(aHist + t * vecb + eb[j], sum[j]);
+                else if (ok && in[j]) X[at(j) + chain_at(t)] = (double)sum[j];
             }
-            __syncthreads();
+            block_sync();
+        }
+        // the chains' last rows change hands, and the middle row
+        const uint32_t mine = aMid + (pass & 1) * vecb;
+        uint32_t peer;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(mine), "r"(side ^ 1));
+#pragma unroll
+        for (int j = 0; j < kE; ++j) {
+            if (!own[j]) continue;
+            const T w = n > 0 ? ldv<T>(aPrev + eb[j]) : T(0);
+            if constexpr (SZ == 4)
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer + eb[j]), "f"((float)w) : "memory");
+            else
+                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(peer + eb[j]), "d"((double)w) : "memory");
+        }
+        __syncwarp();
+        cluster_meet();
+        {
+            const uint32_t R = record();
+#pragma unroll
+            for (int j = 0; j < kE; ++j) {
+                if (!own[j]) continue;
+                T v = T(0);
+                if (in[j]) {
+                    v = nxt[j];
+                    if (n > 0) v -= pair(R + fpair, aPrev, j, nbf);
+                    v -= pair(R + bpair, mine, j, nbb);
+                }
+                sts(aV + eb[j], v);
+            }
+            product(R, sum);
+#pragma unroll
+            for (int j = 0; j < kE; ++j) {
+                if (!own[j]) continue;
+                sts(aPrev + eb[j], sum[j]);
+                if (ok && in[j] && side == 0) X[at(j) + h * ystep] = (double)sum[j];
+            }
+            if (!HIST && n > 0) ahead(X, chain_at(n - 1));
+            block_sync();
+        }
+        // and back: x_y = w_y - S^{-1} (the coupling to the row after)
+        for (int t = n - 1; t >= 0; --t) {
+            const uint32_t R = record();
+#pragma unroll
+            for (int j = 0; j < kE; ++j)
+                if (own[j]) sts(aV + eb[j], in[j] ? pair(R + bpair, aPrev, j, nbb) : T(0));
+            product(R, sum);
+#pragma unroll
+            for (int j = 0; j < kE; ++j) {
+                if (!own[j]) continue;
+                const T x = (HIST ? ldv<T>(aHist + t * vecb + eb[j]) : nxt[j]) - sum[j];
+                sts(aPrev + eb[j], x);
+                if (ok && in[j]) X[at(j) + chain_at(t)] = (double)x;
+            }
+            if (!HIST && t > 0) ahead(X, chain_at(t - 1));
+            block_sync();
         }
     }
 }
 
-int e0_ld(int m) { return (m + 1 + 3) & ~3; }
+// How the solve is launched: threads and groups per tile row, slots and
+// shared memory, and whether the chains' right-hand sides are kept there.
+struct SolvePlan {
+    int threads, P, slots;
+    size_t smem;
+    bool hist;
+};
 
 template <typename T>
-size_t solve_smem(int m) {
-    const int ld = e0_ld(m), nq4 = ld / 4;
-    const int ng = std::max(1, std::min(m + 1, kThreads / nq4));
-    return (size_t)(3 + ng) * kRB * ld * sizeof(T);
+SolvePlan solve_plan(int m, int nSp, int nrhs) {
+    SolvePlan pl{};
+    const int nt = e0_nt(m), bp = 8 * nt, nr = std::min(nrhs, kRB), b = m + 1;
+    pl.P = std::max(1, std::min({nt, e0_threads(nrhs) / (8 * nt), kMaxParts}));
+    pl.threads = (8 * nt * pl.P + 31) / 32 * 32;
+    const size_t rec = e0_record(nt) * sizeof(T);
+    const size_t vec = (size_t)(4 + pl.P) * nr * bp * sizeof(T);
+    const size_t hist = (size_t)(b - 1 - b / 2 > b / 2 ? b - 1 - b / 2 : b / 2) * nr * bp * sizeof(T);
+    // As many blocks per SM as it takes to have every chain resident, at
+    // most 4 (2 in FP64): chains that wait for each other's copies keep HBM
+    // busy, while a second wave would leave half the SMs idle at its end.
+    const int most = sizeof(T) == 4 ? 4 : 2;
+    int per = std::min(most, std::max(1, (2 * nSp + device_sm_count() - 1) / device_sm_count()));
+    for (;; --per) {
+        const size_t room = kSmemPerSm / per - 2048;   // driver's share, alignment, barriers
+        if (vec + rec > room && per > 1) continue;
+        pl.hist = vec + hist + 2 * rec <= room;
+        const size_t left = room - vec - (pl.hist ? hist : 0);
+        pl.slots = (int)std::max<size_t>(1, std::min<size_t>(8, left / rec));
+        pl.smem = pl.slots * rec + vec + (pl.hist ? hist : 0) + 512;   // 512: alignment
+        return pl;
+    }
 }
 
-// the FP32 solve: two staged half blocks and the vectors
-size_t tma_smem(int m) {
-    const size_t ld = e0_ld(m), hb = (m + 2) / 2;
-    return 2 * hb * ld * sizeof(float) + solve_smem<float>(m);
+template <typename T, bool HIST, int NR>
+int solve_launch(cudaStream_t s, const DevSystem& d, const SolvePlan& pl, const T* fac,
+                 const double* B, double* X, int nrhs) {
+    auto kern = k_e0_solve<T, HIST, NR>;
+    // the attribute is per device and per kernel: every call sets the same
+    // value, so none can shrink it under another's launch
+    RTE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerSm));
+    kern<<<2 * d.nSp, pl.threads + 32, pl.smem, s>>>(d.m, d.nSp, nrhs, pl.P, pl.slots, fac, B, X);
+    count_launches(1);
+    RTE_CUDA_TRY(cudaGetLastError());
+    return RTE_OK;
 }
+
+template <typename T, int NR>
+int solve_nr(cudaStream_t s, const DevSystem& d, const SolvePlan& pl, const T* fac, const double* B,
+             double* X, int nrhs) {
+    return pl.hist ? solve_launch<T, true, NR>(s, d, pl, fac, B, X, nrhs)
+                   : solve_launch<T, false, NR>(s, d, pl, fac, B, X, nrhs);
+}
+
+template <typename T>
+int solve(cudaStream_t s, const DevSystem& d, const T* fac, const double* B, double* X, int nrhs) {
+    const SolvePlan pl = solve_plan<T>(d.m, d.nSp, nrhs);
+    switch (std::min(nrhs, kRB)) {
+        case 1: return solve_nr<T, 1>(s, d, pl, fac, B, X, nrhs);
+        case 2: return solve_nr<T, 2>(s, d, pl, fac, B, X, nrhs);
+        case 3: return solve_nr<T, 3>(s, d, pl, fac, B, X, nrhs);
+        default: return solve_nr<T, kRB>(s, d, pl, fac, B, X, nrhs);
+    }
+}
+
+size_t factor_smem(int m) { return (size_t)((m + 1) * (m + 1) + 2 * (m + 1)) * sizeof(double); }
 
 }  // namespace
 
-// m <= 156: the FP32 solve's two staged blocks and vectors fit in 227 KB of
-// shared memory (and the FP64 set-up's Schur complement in 200 KB).
+// m <= 156: the set-up's FP64 Schur complement fits in 200 KB of shared
+// memory (and the solve's record, 113 KB in FP64, beside its vectors).
 bool e0_direct_fits(int m) { return m >= 1 && m <= kMaxM; }
 
 size_t e0_direct_bytes(int m, int nSp, bool fp64) {
-    const size_t ld = e0_ld(m);
-    return (size_t)nSp * (m + 1) * ld * ld * (fp64 ? 8 : 4);
+    return (size_t)nSp * (m + 1) * e0_record(e0_nt(m)) * (fp64 ? 8 : 4);
 }
 
 size_t e0_direct_scratch_bytes(int m, int nSp) {
-    return (size_t)nSp * (m + 1) * (m + 1) * sizeof(double);
-}
-
-// Largest dynamic shared memory of a kernel over every mesh the route takes:
-// the attribute is per device and per kernel, so every call (from any host
-// thread, for any mesh) sets the same value and no call can shrink it under
-// another's launch.
-size_t factor_smem(int m) { return (size_t)((m + 1) * (m + 1) + 2 * (m + 1)) * sizeof(double); }
-template <typename T>
-size_t max_solve_smem() {
-    size_t mx = 0;
-    for (int m = 1; m <= kMaxM; ++m) mx = std::max(mx, solve_smem<T>(m));
-    return mx;
-}
-size_t max_tma_smem() {
-    size_t mx = 0;
-    for (int m = 1; m <= kMaxM; ++m) mx = std::max(mx, tma_smem(m));
-    return mx;
+    return (size_t)nSp * 2 * (m + 1) * (m + 1) * sizeof(double);
 }
 
 int e0_direct_factor(cudaStream_t s, const DevSystem& d, double* scratch, float* out32,
@@ -530,34 +652,21 @@ int e0_direct_factor(cudaStream_t s, const DevSystem& d, double* scratch, float*
     const size_t sm = factor_smem(m);
     RTE_CUDA_TRY(cudaFuncSetAttribute(k_e0_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)factor_smem(kMaxM)));
-    count_launches(1);
-    k_e0_factor<<<d.nSp, kThreads, sm, s>>>(m, d.nSp, e0_ld(m), d.e0coef, scratch, out32, out64);
+    count_launches(2);
+    k_e0_factor<<<dim3(d.nSp, 2), kThreads, sm, s>>>(m, d.nSp, 0, d.e0coef, scratch, out32, out64);
+    k_e0_factor<<<d.nSp, kThreads, sm, s>>>(m, d.nSp, 1, d.e0coef, scratch, out32, out64);
     RTE_CUDA_TRY(cudaGetLastError());
     return RTE_OK;
 }
 
 int e0_direct_solve(cudaStream_t s, const DevSystem& d, const double* B, double* X, int nrhs,
                     bool fp64) {
-    const int m = d.m, ld = e0_ld(m);
     if (fp64) {
         if (!d.e0lu64) return fail(RTE_ERR_ARG, "no FP64 direct E_0 factor");
-        const size_t sm = solve_smem<double>(m);
-        RTE_CUDA_TRY(cudaFuncSetAttribute(k_e0_direct<double>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)max_solve_smem<double>()));
-        k_e0_direct<double><<<d.nSp, kThreads, sm, s>>>(m, d.nSp, nrhs, ld, d.e0lu64, d.e0coef,
-                                                        B, X);
-    } else {
-        if (!d.e0lu32) return fail(RTE_ERR_ARG, "no FP32 direct E_0 factor");
-        const size_t sm = tma_smem(m);
-        RTE_CUDA_TRY(cudaFuncSetAttribute(k_e0_direct_tma,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)max_tma_smem()));
-        k_e0_direct_tma<<<d.nSp, kThreads, sm, s>>>(m, d.nSp, nrhs, ld, d.e0lu32, d.e0coef, B, X);
+        return solve<double>(s, d, d.e0lu64, B, X, nrhs);
     }
-    count_launches(1);
-    RTE_CUDA_TRY(cudaGetLastError());
-    return RTE_OK;
+    if (!d.e0lu32) return fail(RTE_ERR_ARG, "no FP32 direct E_0 factor");
+    return solve<float>(s, d, d.e0lu32, B, X, nrhs);
 }
 
 int e0_direct_error(cudaStream_t s) {
@@ -568,7 +677,7 @@ int e0_direct_error(cudaStream_t s) {
     if (e) {
         const int zero = 0;
         cudaMemcpyToSymbolAsync(g_e0_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-        return fail(RTE_ERR_TIMEOUT, "a wait for a staged E_0 factor block timed out");
+        return fail(RTE_ERR_TIMEOUT, "a wait for a staged E_0 factor record timed out");
     }
     return RTE_OK;
 }

@@ -11,8 +11,8 @@
 //    b is made (the restriction, or the CG update on level 0), prolongation
 //    runs inside the smoothing step after it, the direction update inside the
 //    product E_c p, the r.z sum inside the last smoothing step: with two
-//    sweeps 4 + 5 (L - 1) phases per CG iteration on L levels, against 26
-//    for L = 4 before (now 19), and none for the V-cycle that no further
+//    sweeps 3 + 5 (L - 1) phases per CG iteration on L levels, against 26
+//    for L = 4 before (now 18), and none for the V-cycle that no further
 //    iteration would use;
 //  * short phases: the loads of a phase are independent and issued first; the
 //    d x d products take their operands as 16-byte broadcasts from shared

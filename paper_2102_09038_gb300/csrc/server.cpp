@@ -247,10 +247,11 @@ size_t rte_estimate_bytes(const rte_problem* p, const rte_options* o, int nrhs) 
                              (o->e0_route == RTE_E0_AUTO && m <= 156))
                           : m <= 156;
     if (direct) {
-        // the factor (FP64 in FP64 mode, FP32 otherwise) and its setup scratch
-        const size_t ld = (m + 1 + 3) & ~(size_t)3;
+        // the factor (FP64 in FP64 mode, FP32 otherwise), one record of 8 x 8
+        // tiles and couplings per row, and its setup scratch
+        const size_t nt = (m + 8) / 8, rec = 32 * nt * (nt + 1) + 2 * ((16 * nt + 63) / 64 * 64);
         const bool fp64 = !o || o->precision == RTE_FP64;
-        b += nSp * (m + 1) * ld * ld * (fp64 ? 8 : 4) + nSp * nRp * 8;
+        b += nSp * (m + 1) * rec * (fp64 ? 8 : 4) + nSp * nRp * 8 * 2;
     } else {
         b += 7 * nRp * nSp * 4;                // FP64 kernel's FP32 copy
         b += 7 * nRp * nSp * 4 * 4 / 3;        // multigrid coefficients

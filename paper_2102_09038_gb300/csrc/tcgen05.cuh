@@ -50,16 +50,17 @@ static __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait for the completion of the phase with the given parity.  A
-// phase that is complete already costs one try: the clock and the limit (in
-// global memory) are read only by a wait that has to go on.
+// Bounded wait for the completion of the phase with the given parity.  The
+// limit (in global memory) is read only by a wait that has gone on for a
+// while: its latency would otherwise be part of every wait that does not
+// succeed at once.
 static __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
-    const long long lim = g_tc_wait_cycles;
     while (true) {
-        if (mbar_try(bar, parity)) return true;
-        if (clock64() - t0 > lim) {
+        for (int i = 0; i < 64; ++i)
+            if (mbar_try(bar, parity)) return true;
+        if (clock64() - t0 > g_tc_wait_cycles) {
             atomicExch(&g_tc_error, 1);
             return false;
         }
