@@ -68,6 +68,8 @@ struct DevSystem {
     const double* Sm;          // [nSm][nSm]
     const double* Vm;          // [nSm][nSm]  eigenvectors of (S^-, M_S^-) as columns
     const double* VmT;         // [nSm][nSm]
+    const double* Wg;          // [2 nSp][nSm] W = [A_1 A_2]^T V, row 2k + d (eigenbasis route)
+    const double* WgT;         // [nSm][2 nSp]
     const double* lamM;        // [nSm]       non-increasing
     const double* WmN;         // [nSm][dM]
     const double* WmNT;        // [dM][nSm]
@@ -97,6 +99,10 @@ struct DevSystem {
     const int* ex_VmT;
     const void* sl_Vm;
     const int* ex_Vm;
+    const void* sl_Wg;         // W and W^T (eigenbasis route)
+    const int* ex_Wg;
+    const void* sl_WgT;
+    const int* ex_WgT;
     const void* sl_Sp;
     const int* ex_Sp;
     const void* sl_Sm;         // S^- (the PCG route's K^- in the mixed modes)
@@ -130,10 +136,19 @@ void gemm_f64(cudaStream_t s, int M, int N, int K, const double* A, int lda,
 void apply_A(cudaStream_t s, const DevSystem& d, const double* U, double* Z,
              int nrhs);
 
+// The eigenbasis route's E between spatial derivatives (kernels.cu): G[r, j,
+// 2k + d] = sign (D_d U_r)[j, k] (nrhs x nRm x 2 nSp), and Y = sum_d D_d^T G_d +
+// M^+ X + R X - M_s^+ V - Q (V, Q may be null).
+void apply_grad(cudaStream_t s, const DevSystem& d, const double* U, double* G, int nrhs,
+                double sign = 1.0);
+void apply_even_grad(cudaStream_t s, const DevSystem& d, const double* G, const double* X,
+                     const double* V, const double* Q, double* Y, int nrhs);
+// The mixed modes' A u (BF16 or FP32 result) and A^T z + M^+ x + R x - M_s^+ v
+// (V may be null) on three odd values per direction, in FP32.
 void apply_A_lo(cudaStream_t s, const DevSystem& d, const float* U, void* Z, bool bf16,
                 int nrhs);
 void apply_even_lo(cudaStream_t s, const DevSystem& d, const float* Zp, const float* X,
-                   const float* V, float* Y, int nrhs, int flags);
+                   const float* V, float* Y, int nrhs);
 void dot_per_rhs(cudaStream_t s, const float* x, const float* y, size_t len, int nrhs,
                  double* partial, double* out);
 void axpby_per_rhs(cudaStream_t s, const float* x, float* y, size_t len, int nrhs,

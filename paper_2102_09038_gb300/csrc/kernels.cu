@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cstdint>
 
 #include "device.h"
 #include "rte_internal.h"
@@ -90,93 +91,6 @@ k_gemm_f64(int M, int N, int K, const double* __restrict__ A, int lda,
             if (beta != 0.0) v += beta * *dst;
             *dst = v;
         }
-    }
-}
-
-// ----------------------------------------------------- transport A (a1)
-// Z[r, j, 3k+c] = sum_n A_n(k, c) (D_n U_r)[j, k]; computed in TC, read as TIn,
-// written as TOut (FP64, or FP32 in / BF16-or-FP32 out for the mixed paths)
-template <typename TIn, typename TOut, typename TC>
-__global__ void k_apply_A(int nRm, int nRp, int nSp, int nrhs,
-                          const int* __restrict__ cell_nodes,
-                          const TC* __restrict__ cell_D,
-                          const TC* __restrict__ A1,
-                          const TC* __restrict__ A2,
-                          const TIn* __restrict__ U, TOut* __restrict__ Z) {
-    const unsigned total = (unsigned)nrhs * nRm * nSp;
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += gridDim.x * blockDim.x) {
-        const int k = (int)(e % (unsigned)nSp);
-        const unsigned rj = e / (unsigned)nSp;
-        const int j = (int)(rj % (unsigned)nRm);
-        const int r = (int)(rj / (unsigned)nRm);
-        const TIn* Ur = U + (size_t)r * nRp * nSp;
-        TC g1 = 0, g2 = 0;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const TC u = static_cast<TC>(Ur[(size_t)cell_nodes[3 * j + a] * nSp + k]);
-            g1 = fma(cell_D[6 * j + a], u, g1);
-            g2 = fma(cell_D[6 * j + 3 + a], u, g2);
-        }
-        TOut* z = Z + rj * (3 * (size_t)nSp) + 3 * k;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) z[c] = static_cast<TOut>(A1[3 * k + c] * g1 + A2[3 * k + c] * g2);
-    }
-}
-
-// ------------------------------------------ A^T + M^+ + R - K^+ (a2, b2)
-template <typename T>
-__global__ void k_apply_even(int nRm, int nRp, int nSp, int nrhs, int nnz,
-                             int flags, const int* __restrict__ adj_ptr,
-                             const int* __restrict__ adj_cell,
-                             const int* __restrict__ adj_loc,
-                             const T* __restrict__ cell_D,
-                             const T* __restrict__ A1,
-                             const T* __restrict__ A2,
-                             const int* __restrict__ st_ptr,
-                             const int* __restrict__ st_col,
-                             const T* __restrict__ sval,
-                             const T* __restrict__ m,
-                             const T* __restrict__ omx,
-                             const T* __restrict__ omy,
-                             const T* __restrict__ Zp,
-                             const T* __restrict__ X,
-                             const T* __restrict__ V, T* __restrict__ Y) {
-    const unsigned total = (unsigned)nrhs * nRp * nSp;
-    const T* Mt = sval + (size_t)kMt * nnz;
-    const T* Ms = sval + (size_t)kMs * nnz;
-    const T* Bx = sval + (size_t)kBx * nnz;
-    const T* By = sval + (size_t)kBy * nnz;
-    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += gridDim.x * blockDim.x) {
-        const int k = (int)(e % (unsigned)nSp);
-        const unsigned ri = e / (unsigned)nSp;
-        const int i = (int)(ri % (unsigned)nRp);
-        const int r = (int)(ri / (unsigned)nRp);
-        T acc = 0;
-        if (flags & 1) {
-            const T a1[3] = {A1[3 * k], A1[3 * k + 1], A1[3 * k + 2]};
-            const T a2[3] = {A2[3 * k], A2[3 * k + 1], A2[3 * k + 2]};
-            const T* Zr = Zp + (size_t)r * nRm * 3 * nSp;
-            for (int p = adj_ptr[i]; p < adj_ptr[i + 1]; ++p) {
-                const int j = adj_cell[p], a = adj_loc[p];
-                const T* z = Zr + (size_t)j * 3 * nSp + 3 * k;
-                const T t1 = a1[0] * z[0] + a1[1] * z[1] + a1[2] * z[2];
-                const T t2 = a2[0] * z[0] + a2[1] * z[1] + a2[2] * z[2];
-                acc += cell_D[6 * j + a] * t1 + cell_D[6 * j + 3 + a] * t2;
-            }
-        }
-        if (flags & 6) {
-            const T mk = m[k], ox = omx[k], oy = omy[k];
-            const T* Xr = X + (size_t)r * nRp * nSp;
-            const T* Vr = V ? V + (size_t)r * nRp * nSp : nullptr;
-            for (int p = st_ptr[i]; p < st_ptr[i + 1]; ++p) {
-                const size_t col = (size_t)st_col[p] * nSp + k;
-                if (flags & 2) acc += (mk * Mt[p] + ox * Bx[p] + oy * By[p]) * Xr[col];
-                if (flags & 4) acc -= Ms[p] * Vr[col];
-            }
-        }
-        Y[e] = acc;
     }
 }
 
@@ -593,7 +507,355 @@ __global__ void k_apply_even_s(int m, int nSp, int nrhs, int flags,
     }
 }
 
+// ------------------------------------------- the eigenbasis route's E
+// (M^- - K^-)^{-1} between A and A^T needs only what A's odd values carry:
+// A u = A_1 (x) D_1 u + A_2 (x) D_2 u has two spatial derivatives per cell and
+// direction, not three free values, and A^T takes two projections back.  So
+// with W = [A_1 A_2]^T V (2 n_S^+ x n_S^-, V the eigenvectors) the
+// contractions run from and to the derivatives, 2/3 of their work, and the
+// two kernels below need 8 products per square, direction and node where A
+// and A^T on three odd values took 12 and 48.
+//
+// W consecutive directions per thread: 2 where the pointers are aligned for it,
+// else 1.
+template <typename T, int N>
+struct alignas(sizeof(T) * N) Pack {
+    T v[N];
+};
+
+// G[r, j, 2k + d] = sign (D_d U_r)[j, k] for both cells of every square.  On
+// the "/"-mesh each hat function of a cell has a derivative along x or along y
+// only, but for one: the terms that are zero are left out.
+template <int W>
+__global__ void __launch_bounds__(256)
+k_grad(int m, int nSp, int nrhs, double sign, const double* __restrict__ cell_D,
+       const double* __restrict__ U, double* __restrict__ G) {
+    const unsigned nk = (unsigned)nSp / W, total = (unsigned)nrhs * m * m * nk;
+    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int k = (int)(e % nk) * W;
+    const unsigned rq = e / nk;
+    const int q = (int)(rq % (unsigned)(m * m)), r = (int)(rq / (unsigned)(m * m));
+    const int I = q % m, J = q / m;
+    const size_t n00 = ((size_t)r * (m + 1) * (m + 1) + (size_t)J * (m + 1) + I) * nSp + k;
+    using PI = Pack<double, W>;
+    auto node = [&](size_t o) { return *reinterpret_cast<const PI*>(U + o); };
+    const PI u00 = node(n00), u10 = node(n00 + nSp), u01 = node(n00 + (size_t)(m + 1) * nSp),
+             u11 = node(n00 + (size_t)(m + 2) * nSp);
+    const double *lo = cell_D + 12 * (size_t)q, *up = lo + 6;   // D_1 of the three vertices, then D_2
+    Pack<double, 2 * W> a, b;
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const double x00 = u00.v[i], x10 = u10.v[i], x01 = u01.v[i], x11 = u11.v[i];
+        a.v[2 * i] = sign * fma(lo[0], x00, lo[1] * x10);
+        a.v[2 * i + 1] = sign * fma(lo[4], x10, lo[5] * x11);
+        b.v[2 * i] = sign * fma(up[1], x11, up[2] * x01);
+        b.v[2 * i + 1] = sign * fma(up[3], x00, up[5] * x01);
+    }
+    double* g = G + ((size_t)rq * 2 * nSp + k) * 2;
+    *reinterpret_cast<Pack<double, 2 * W>*>(g) = a;
+    *reinterpret_cast<Pack<double, 2 * W>*>(g + 2 * (size_t)nSp) = b;
+}
+
+// Y = sum_d D_d^T G_d + [M^+ X + R X] - [M_s^+ V] - [Q] (the terms whose
+// pointer is set), G as k_grad lays it out.  The stencil sums come before the
+// direction's factors, and the boundary terms on boundary nodes alone.
+template <int W>
+__global__ void __launch_bounds__(256)
+k_even_grad(int m, int nSp, int nrhs, const double* __restrict__ cell_D, const double* __restrict__ ell4,
+            const double* __restrict__ mk, const double* __restrict__ omx, const double* __restrict__ omy,
+            const double* __restrict__ G, const double* __restrict__ X, const double* __restrict__ V,
+            const double* __restrict__ Q, double* __restrict__ Y) {
+    const int n1 = m + 1, nRp = n1 * n1;
+    const unsigned nk = (unsigned)nSp / W, total = (unsigned)nrhs * nRp * nk;
+    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int k = (int)(e % nk) * W;
+    const unsigned ri = e / nk;
+    const int i = (int)(ri % (unsigned)nRp), r = (int)(ri / (unsigned)nRp);
+    const int y = i / n1, x = i - y * n1;
+    using P = Pack<double, W>;
+    auto at = [&](const double* p, int node) {
+        return *reinterpret_cast<const P*>(p + ((size_t)r * nRp + node) * nSp + k);
+    };
+    double acc[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) acc[w] = 0.0;
+    // the six cells around the node: square, cell of the square, and which of
+    // the two derivatives the node's hat function has there
+    const double* Gr = G + (size_t)r * 4 * m * m * nSp + 2 * k;
+    auto cell = [&](int I, int J, int up, int loc, bool d1, bool d2) {
+        const int j = 2 * (J * m + I) + up;
+        const Pack<double, 2 * W> g = *reinterpret_cast<const Pack<double, 2 * W>*>(Gr + (size_t)j * 2 * nSp);
+        const double* D = cell_D + 6 * (size_t)j + loc;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            if (d1) acc[w] = fma(D[0], g.v[2 * w], acc[w]);
+            if (d2) acc[w] = fma(D[3], g.v[2 * w + 1], acc[w]);
+        }
+    };
+    const bool l = x > 0, rt = x < m, dn = y > 0, tp = y < m;
+    if (rt && tp) {
+        cell(x, y, 0, 0, true, false);
+        cell(x, y, 1, 0, false, true);
+    }
+    if (l && tp) cell(x - 1, y, 0, 1, true, true);
+    if (l && dn) {
+        cell(x - 1, y - 1, 0, 2, false, true);
+        cell(x - 1, y - 1, 1, 1, true, false);
+    }
+    if (rt && dn) cell(x, y - 1, 1, 2, true, true);
+    // neighbours in the order of the ELL form; one outside takes the node
+    // itself (its coefficient is zero)
+    const int nb[7] = {i, rt ? i + 1 : i, l ? i - 1 : i, tp ? i + n1 : i, dn ? i - n1 : i,
+                       rt && tp ? i + n1 + 1 : i, l && dn ? i - n1 - 1 : i};
+    const size_t sl = (size_t)7 * nRp;
+    if (X) {
+        double mass[W], bx[W], by[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) mass[w] = bx[w] = by[w] = 0.0;
+        const bool edge = !(l && rt && dn && tp);
+#pragma unroll
+        for (int dir = 0; dir < 7; ++dir) {
+            const size_t pe = (size_t)dir * nRp + i;
+            const P u = at(X, nb[dir]);
+            const double c = ell4[pe];
+#pragma unroll
+            for (int w = 0; w < W; ++w) mass[w] = fma(c, u.v[w], mass[w]);
+            if (edge) {
+                const double cx = ell4[2 * sl + pe], cy = ell4[3 * sl + pe];
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    bx[w] = fma(cx, u.v[w], bx[w]);
+                    by[w] = fma(cy, u.v[w], by[w]);
+                }
+            }
+        }
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            acc[w] = fma(mk[k + w], mass[w], acc[w]);
+            if (edge) acc[w] = fma(omx[k + w], bx[w], fma(omy[k + w], by[w], acc[w]));
+        }
+    }
+    if (V) {
+#pragma unroll
+        for (int dir = 0; dir < 7; ++dir) {
+            const P v = at(V, nb[dir]);
+            const double c = -ell4[sl + (size_t)dir * nRp + i];
+#pragma unroll
+            for (int w = 0; w < W; ++w) acc[w] = fma(c, v.v[w], acc[w]);
+        }
+    }
+    const size_t o = (size_t)ri * nSp + k;
+    P out;
+    if (Q) {
+        const P q = *reinterpret_cast<const P*>(Q + o);
+#pragma unroll
+        for (int w = 0; w < W; ++w) out.v[w] = acc[w] - q.v[w];
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) out.v[w] = acc[w];
+    }
+    *reinterpret_cast<P*>(Y + o) = out;
+}
+
+// ------------------------------------------- the mixed modes' inner E
+// A u and A^T z + M^+ x + R x - M_s^+ v on three odd values per direction, in
+// FP32: between the derivatives instead (as above) the BF16 or TF32 operands
+// of the contractions lose three to four times as much on smooth fields (7.5e-2
+// against 1.9e-2 of E u on a 128 x 128 solution in BF16).  Bound by memory
+// once a thread takes four directions (16-byte accesses, the cell and stencil
+// coefficients loaded once for four) and leaves out the derivatives that are
+// zero.  Measured on 128 x 128 / 256 directions: A u 56 us before, 19 now, the gather 94
+// before, 50 now.
+template <typename TOut>
+__global__ void __launch_bounds__(256)
+k_odd_lo(int m, int nSp, int nrhs, const float* __restrict__ cell_D, const float* __restrict__ A1,
+         const float* __restrict__ A2, const float* __restrict__ U, TOut* __restrict__ Z) {
+    const unsigned nk = (unsigned)nSp / 4, total = (unsigned)nrhs * m * m * nk;
+    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int k = (int)(e % nk) * 4;
+    const unsigned rq = e / nk;
+    const int q = (int)(rq % (unsigned)(m * m)), r = (int)(rq / (unsigned)(m * m));
+    const int I = q % m, J = q / m;
+    const size_t n00 = ((size_t)r * (m + 1) * (m + 1) + (size_t)J * (m + 1) + I) * nSp + k;
+    using P4 = Pack<float, 4>;
+    auto node = [&](size_t o) { return *reinterpret_cast<const P4*>(U + o); };
+    const P4 u00 = node(n00), u10 = node(n00 + nSp), u01 = node(n00 + (size_t)(m + 1) * nSp),
+             u11 = node(n00 + (size_t)(m + 2) * nSp);
+    float a1[12], a2[12];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        *reinterpret_cast<P4*>(a1 + 4 * i) = *reinterpret_cast<const P4*>(A1 + 3 * k + 4 * i);
+        *reinterpret_cast<P4*>(a2 + 4 * i) = *reinterpret_cast<const P4*>(A2 + 3 * k + 4 * i);
+    }
+    const float *lo = cell_D + 12 * (size_t)q, *up = lo + 6;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        float z[12];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float g1 = c == 0 ? fmaf(lo[0], u00.v[i], lo[1] * u10.v[i])
+                                    : fmaf(up[1], u11.v[i], up[2] * u01.v[i]);
+            const float g2 = c == 0 ? fmaf(lo[4], u10.v[i], lo[5] * u11.v[i])
+                                    : fmaf(up[3], u00.v[i], up[5] * u01.v[i]);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) z[3 * i + j] = a1[3 * i + j] * g1 + a2[3 * i + j] * g2;
+        }
+        TOut* out = Z + ((size_t)rq * 2 + c) * 3 * nSp + 3 * k;
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            Pack<TOut, 4> w;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w.v[i] = static_cast<TOut>(z[4 * p + i]);
+            *reinterpret_cast<Pack<TOut, 4>*>(out + 4 * p) = w;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256)
+k_even_lo(int m, int nSp, int nrhs, const float* __restrict__ cell_D, const float* __restrict__ A1,
+          const float* __restrict__ A2, const float* __restrict__ ell4,
+          const float* __restrict__ mk, const float* __restrict__ omx,
+          const float* __restrict__ omy, const float* __restrict__ Z, const float* __restrict__ X,
+          const float* __restrict__ V, float* __restrict__ Y) {
+    const int n1 = m + 1, nRp = n1 * n1;
+    const unsigned nk = (unsigned)nSp / 4, total = (unsigned)nrhs * nRp * nk;
+    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= total) return;
+    const int k = (int)(e % nk) * 4;
+    const unsigned ri = e / nk;
+    const int i = (int)(ri % (unsigned)nRp), r = (int)(ri / (unsigned)nRp);
+    const int y = i / n1, x = i - y * n1;
+    using P4 = Pack<float, 4>;
+    auto at = [&](const float* p, int node) {
+        return *reinterpret_cast<const P4*>(p + ((size_t)r * nRp + node) * nSp + k);
+    };
+    float acc[4] = {0.f, 0.f, 0.f, 0.f}, a1[12], a2[12];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        *reinterpret_cast<P4*>(a1 + 4 * p) = *reinterpret_cast<const P4*>(A1 + 3 * k + 4 * p);
+        *reinterpret_cast<P4*>(a2 + 4 * p) = *reinterpret_cast<const P4*>(A2 + 3 * k + 4 * p);
+    }
+    const float* Zr = Z + (size_t)r * 6 * m * m * nSp + 3 * k;
+    auto cell = [&](int I, int J, int up, int loc, bool d1, bool d2) {
+        const int j = 2 * (J * m + I) + up;
+        const float* zp = Zr + (size_t)j * 3 * nSp;
+        float z[12];
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+            *reinterpret_cast<P4*>(z + 4 * p) = *reinterpret_cast<const P4*>(zp + 4 * p);
+        const float* D = cell_D + 6 * (size_t)j + loc;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if (d1)
+                acc[w] = fmaf(D[0], a1[3 * w] * z[3 * w] + a1[3 * w + 1] * z[3 * w + 1] + a1[3 * w + 2] * z[3 * w + 2], acc[w]);
+            if (d2)
+                acc[w] = fmaf(D[3], a2[3 * w] * z[3 * w] + a2[3 * w + 1] * z[3 * w + 1] + a2[3 * w + 2] * z[3 * w + 2], acc[w]);
+        }
+    };
+    const bool l = x > 0, rt = x < m, dn = y > 0, tp = y < m;
+    if (rt && tp) {
+        cell(x, y, 0, 0, true, false);
+        cell(x, y, 1, 0, false, true);
+    }
+    if (l && tp) cell(x - 1, y, 0, 1, true, true);
+    if (l && dn) {
+        cell(x - 1, y - 1, 0, 2, false, true);
+        cell(x - 1, y - 1, 1, 1, true, false);
+    }
+    if (rt && dn) cell(x, y - 1, 1, 2, true, true);
+    const int nb[7] = {i, rt ? i + 1 : i, l ? i - 1 : i, tp ? i + n1 : i, dn ? i - n1 : i,
+                       rt && tp ? i + n1 + 1 : i, l && dn ? i - n1 - 1 : i};
+    const size_t sl = (size_t)7 * nRp;
+    const bool edge = !(l && rt && dn && tp);
+    float mass[4] = {0.f, 0.f, 0.f, 0.f}, bx[4] = {0.f, 0.f, 0.f, 0.f}, by[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int dir = 0; dir < 7; ++dir) {
+        const size_t pe = (size_t)dir * nRp + i;
+        const P4 u = at(X, nb[dir]);
+        const float c = ell4[pe];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) mass[w] = fmaf(c, u.v[w], mass[w]);
+        if (edge) {
+            const float cx = ell4[2 * sl + pe], cy = ell4[3 * sl + pe];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                bx[w] = fmaf(cx, u.v[w], bx[w]);
+                by[w] = fmaf(cy, u.v[w], by[w]);
+            }
+        }
+        if (V) {
+            const P4 v = at(V, nb[dir]);
+            const float cs = -ell4[sl + pe];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) acc[w] = fmaf(cs, v.v[w], acc[w]);
+        }
+    }
+    P4 out;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+        acc[w] = fmaf(mk[k + w], mass[w], acc[w]);
+        if (edge) acc[w] = fmaf(omx[k + w], bx[w], fmaf(omy[k + w], by[w], acc[w]));
+        out.v[w] = acc[w];
+    }
+    *reinterpret_cast<P4*>(Y + (size_t)ri * nSp + k) = out;
+}
+
+// whether pointers allow W = 2 accesses of T (null ones do)
+template <typename T, typename... Ps>
+bool paired(const Ps*... p) {
+    return (((reinterpret_cast<uintptr_t>(p) & (2 * sizeof(T) - 1)) == 0) && ...);
+}
+
 }  // namespace
+
+void apply_grad(cudaStream_t s, const DevSystem& d, const double* U, double* G, int nrhs,
+                double sign) {
+    // G is the library's own work array: aligned for four values
+    const bool two = paired<double>(U);
+    const size_t total = (size_t)nrhs * d.m * d.m * (d.nSp / (two ? 2 : 1));
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    count_launches(1);
+    if (two) k_grad<2><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, sign, d.cell_D, U, G);
+    else k_grad<1><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, sign, d.cell_D, U, G);
+}
+
+void apply_even_grad(cudaStream_t s, const DevSystem& d, const double* G, const double* X,
+                     const double* V, const double* Q, double* Y, int nrhs) {
+    const bool two = paired<double>(X, V, Q, Y);
+    const size_t total = (size_t)nrhs * d.nRp * (d.nSp / (two ? 2 : 1));
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    count_launches(1);
+    if (two)
+        k_even_grad<2><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.cell_D, d.ell4, d.ang_m, d.ang_omx,
+                                              d.ang_omy, G, X, V, Q, Y);
+    else
+        k_even_grad<1><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.cell_D, d.ell4, d.ang_m, d.ang_omx,
+                                              d.ang_omy, G, X, V, Q, Y);
+}
+
+void apply_A_lo(cudaStream_t s, const DevSystem& d, const float* U, void* Z, bool bf16, int nrhs) {
+    const size_t total = (size_t)nrhs * d.m * d.m * (d.nSp / 4);
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    count_launches(1);
+    if (bf16)
+        k_odd_lo<__nv_bfloat16><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U,
+                                                       static_cast<__nv_bfloat16*>(Z));
+    else
+        k_odd_lo<float><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U,
+                                               static_cast<float*>(Z));
+}
+
+void apply_even_lo(cudaStream_t s, const DevSystem& d, const float* Zp, const float* X,
+                   const float* V, float* Y, int nrhs) {
+    const size_t total = (size_t)nrhs * d.nRp * (d.nSp / 4);
+    count_launches(1);
+    k_even_lo<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
+        d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, d.lo.ell4, d.lo.m, d.lo.omx, d.lo.omy, Zp,
+        X, V, Y);
+}
 
 static std::atomic<long long> g_launches{0};
 void count_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
@@ -628,18 +890,6 @@ void apply_A(cudaStream_t s, const DevSystem& d, const double* U, double* Z, int
         d.m, d.nSp, nrhs, d.cell_D, d.ang_A1, d.ang_A2, U, Z);
 }
 
-void apply_A_lo(cudaStream_t s, const DevSystem& d, const float* U, void* Z, bool bf16,
-                int nrhs) {
-    const size_t total = (size_t)nrhs * d.nRm * d.nSp;
-    count_launches(1);
-    if (bf16)
-        k_apply_A_s<float, __nv_bfloat16, float><<<grid_for(total, d.tpb_A), d.tpb_A, 0, s>>>(
-            d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U, static_cast<__nv_bfloat16*>(Z));
-    else
-        k_apply_A_s<float, float, float><<<grid_for(total, d.tpb_A), d.tpb_A, 0, s>>>(
-            d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U, static_cast<float*>(Z));
-}
-
 void apply_even(cudaStream_t s, const DevSystem& d, const double* Zp, const double* X,
                 const double* V, double* Y, int nrhs, int flags) {
     const size_t total = (size_t)nrhs * d.nRp * d.nSp;
@@ -647,15 +897,6 @@ void apply_even(cudaStream_t s, const DevSystem& d, const double* Zp, const doub
     k_apply_even_s<double><<<grid_for(total, d.tpb_even), d.tpb_even, 0, s>>>(
         d.m, d.nSp, nrhs, flags, d.cell_D, d.ang_A1, d.ang_A2, d.ell4, d.ang_m, d.ang_omx,
         d.ang_omy, Zp, X, V, Y);
-}
-
-void apply_even_lo(cudaStream_t s, const DevSystem& d, const float* Zp, const float* X,
-                   const float* V, float* Y, int nrhs, int flags) {
-    const size_t total = (size_t)nrhs * d.nRp * d.nSp;
-    count_launches(1);
-    k_apply_even_s<float><<<grid_for(total, d.tpb_even), d.tpb_even, 0, s>>>(
-        d.m, d.nSp, nrhs, flags, d.lo.cell_D, d.lo.A1, d.lo.A2, d.lo.ell4, d.lo.m, d.lo.omx,
-        d.lo.omy, Zp, X, V, Y);
 }
 
 void mk_combine(cudaStream_t s, const DevSystem& d, const double* Z, const double* G,

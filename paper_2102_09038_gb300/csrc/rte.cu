@@ -979,6 +979,53 @@ int mk_inv_eigen(rte_handle* h, const double* Z1, double* Z2, int nrhs) {
     return RTE_OK;
 }
 
+// The same between spatial derivatives (kernels.cu: k_grad): with Z1 = A u
+// given by G = [D_1 u, D_2 u], first = G W 1/(at - lam as); T = first W^T are
+// A^T's projections of the result, or Z = first V^T the odd values themselves.
+int mk_first(rte_handle* h, const double* G, int nrhs) {
+    const DevSystem& d = h->d;
+    const int rows = nrhs * d.nRm, n2 = 2 * d.nSp;
+    if (d.split_S > 0) {
+        const int S = split_slices_now(h);
+        int* ea = nullptr;
+        {
+            Scope sc(h, "split_digits");
+            RTE_TRY(ozaki_split(h->stream, G, rows, n2, S, h->slices, &ea));
+        }
+        {
+            Scope sc(h, "dgemm_split_mk1");
+            RTE_TRY(ozaki_gemm(h->stream, h->slices, ea, rows, d.sl_WgT, d.ex_WgT, d.nSm, n2, S,
+                               h->z4, d.nSm, 1, d.mk_rinv, d.nRm, d.split_S));
+        }
+        return RTE_OK;
+    }
+    Scope sc(h, "gemm_mk_eig1");
+    gemm_f64(h->stream, rows, d.nSm, n2, G, n2, d.Wg, d.nSm, h->z4, d.nSm, 1.0, 0.0, 1, d.cell_at,
+             d.cell_as, d.lamM, d.nRm);
+    return RTE_OK;
+}
+
+// odd: Z = first V^T (rows x nSm), else T = first W^T (rows x 2 nSp)
+int mk_second(rte_handle* h, double* out, int nrhs, bool odd) {
+    const DevSystem& d = h->d;
+    const int rows = nrhs * d.nRm, N = odd ? d.nSm : 2 * d.nSp;
+    if (d.split_S > 0) {
+        const int S = split_slices_now(h);
+        int* ea = nullptr;
+        {
+            Scope sc(h, "split_digits");
+            RTE_TRY(ozaki_split(h->stream, h->z4, rows, d.nSm, S, h->slices, &ea));
+        }
+        Scope sc(h, "dgemm_split_mk2");
+        return ozaki_gemm(h->stream, h->slices, ea, rows, odd ? d.sl_Vm : d.sl_Wg,
+                          odd ? d.ex_Vm : d.ex_Wg, N, d.nSm, S, out, N, 0, nullptr, 1, d.split_S);
+    }
+    Scope sc(h, "gemm_mk_eig2");
+    gemm_f64(h->stream, rows, N, d.nSm, h->z4, d.nSm, odd ? d.VmT : d.WgT, N, out, N, 1.0, 0.0, 0,
+             nullptr, nullptr, nullptr, 1);
+    return RTE_OK;
+}
+
 // x = (M^- - K^-_N)^{-1} b by eq. (MmKprecond):
 // x = ((b W_N) .* (F - 1/at)) W_N^T + (b M_S^{-1}) / at
 int mk_prec(rte_handle* h, const double* B, double* X, double* tmp, int nrhs) {
@@ -1177,14 +1224,23 @@ int mk_inv(rte_handle* h, const double* Z1, double* Z2, int nrhs) {
     return mk_inv_eigen(h, Z1, Z2, nrhs);
 }
 
-// y = E x (with_k: y = (E - K^+) x).  Uses z1, z2 (and z3, z4 for routes).
-int apply_E(rte_handle* h, const double* x, double* y, int nrhs, bool with_k) {
+// y = E x (with_k: y = (E - K^+) x; sub set: y = that - sub).  Uses z1, z2
+// (and z3, z4 for routes).
+int apply_E(rte_handle* h, const double* x, double* y, int nrhs, bool with_k,
+            const double* sub = nullptr) {
     const DevSystem& d = h->d;
+    const bool eigen = h->opt.mk_route != RTE_MK_PCG;
     {
         Scope sc(h, "transport_A");
-        apply_A(h->stream, d, x, h->z1, nrhs);
+        if (eigen) apply_grad(h->stream, d, x, h->z1, nrhs);
+        else apply_A(h->stream, d, x, h->z1, nrhs);
     }
-    RTE_TRY(mk_inv(h, h->z1, h->z2, nrhs));
+    if (eigen) {
+        RTE_TRY(mk_first(h, h->z1, nrhs));
+        RTE_TRY(mk_second(h, h->z2, nrhs, false));
+    } else {
+        RTE_TRY(mk_inv(h, h->z1, h->z2, nrhs));
+    }
     double* V = nullptr;
     if (with_k) {
         V = h->e8;
@@ -1202,7 +1258,13 @@ int apply_E(rte_handle* h, const double* x, double* y, int nrhs, bool with_k) {
         }
     }
     Scope sc(h, "apply_even");
-    apply_even(h->stream, d, h->z2, x, V, y, nrhs, with_k ? 7 : 3);
+    if (eigen) {
+        apply_even_grad(h->stream, d, h->z2, x, V, sub, y, nrhs);
+    } else {
+        apply_even(h->stream, d, h->z2, x, V, y, nrhs, with_k ? 7 : 3);
+        if (sub)
+            axpby_per_rhs(h->stream, sub, y, (size_t)d.nRp * d.nSp, nrhs, nullptr, -1.0, nullptr, 1.0);
+    }
     return RTE_OK;
 }
 
@@ -1252,7 +1314,7 @@ int apply_E_lo(rte_handle* h, const float* x, float* y, int nrhs, bool with_k) {
         RTE_TRY(tc_gemm(h->stream, k));
     }
     Scope sc(h, "apply_even_lo");
-    apply_even_lo(h->stream, d, h->zf, x, V, y, nrhs, with_k ? 7 : 3);
+    apply_even_lo(h->stream, d, h->zf, x, V, y, nrhs);
     return RTE_OK;
 }
 
@@ -1721,6 +1783,22 @@ int rte_setup(const rte_problem* prob, const rte_options* opts, void* stream,
         }
     UP(Vm, Vm);
     UP(VmT, VmT);
+    // W = [A_1 A_2]^T V and its transpose: the eigenbasis seen from the
+    // spatial derivatives (row 2k + d: derivative d, direction k)
+    std::vector<double> Wg((size_t)2 * n * nm), WgT((size_t)2 * n * nm);
+    if (o.mk_route != RTE_MK_PCG) {
+        for (int k = 0; k < n; ++k)
+            for (int dd = 0; dd < 2; ++dd) {
+                const double* a = (dd == 0 ? hs.A1.data() : hs.A2.data()) + 3 * k;
+                const double* v = &Vm[(size_t)3 * k * nm];
+                double* w = &Wg[(size_t)(2 * k + dd) * nm];
+                for (int t = 0; t < nm; ++t) w[t] = a[0] * v[t] + a[1] * v[nm + t] + a[2] * v[2 * nm + t];
+            }
+        for (int x = 0; x < 2 * n; ++x)
+            for (int t = 0; t < nm; ++t) WgT[(size_t)t * 2 * n + x] = Wg[(size_t)x * nm + t];
+        UP(Wg, Wg);
+        UP(WgT, WgT);
+    }
     UP(lamM, h->h_lamM);
     UP(WmN, WmN);
     UP(WmNT, WmNT);
@@ -1932,13 +2010,16 @@ int rte_setup(const rte_problem* prob, const rte_options* opts, void* stream,
                 return bail(fail(RTE_ERR_ARG, "split_slices must be in [1, 9]"));
             d.split_S = o.split_slices;
             struct Src { const double* m; int rows, K; const void** sl; const int** ex; };
-            Src srcs[4] = {{d.VmT, nm, nm, &d.sl_VmT, &d.ex_VmT},
+            Src srcs[6] = {{d.VmT, nm, nm, &d.sl_VmT, &d.ex_VmT},
                            {d.Vm, nm, nm, &d.sl_Vm, &d.ex_Vm},
+                           {d.WgT, nm, 2 * n, &d.sl_WgT, &d.ex_WgT},
+                           {d.Wg, 2 * n, nm, &d.sl_Wg, &d.ex_Wg},
                            {d.Sp, n, n, &d.sl_Sp, &d.ex_Sp},
                            {d.Sm, nm, nm, &d.sl_Sm, &d.ex_Sm}};
             for (auto& sr : srcs) {
                 // S^- is needed as a GEMM operand only by the PCG route
                 if (sr.m == d.Sm && o.mk_route != RTE_MK_PCG) continue;
+                if ((sr.m == d.Wg || sr.m == d.WgT) && o.mk_route == RTE_MK_PCG) continue;
                 char* p = nullptr;
                 rc = dalloc(h, &p, ozaki_slice_bytes(sr.rows, sr.K, d.split_S));
                 if (rc) return bail(rc);
@@ -2190,6 +2271,13 @@ int rte_odd(rte_handle* h, const double* u_plus, const double* l_minus, double* 
     const DevSystem& d = h->d;
     cudaStream_t s = h->stream;
     const size_t len = (size_t)d.nRm * d.nSm;
+    if (!l_minus && h->opt.mk_route != RTE_MK_PCG) {
+        apply_grad(s, d, u_plus, h->z1, nrhs, -1.0);   // -[D_1 u, D_2 u]
+        RTE_TRY(mk_first(h, h->z1, nrhs));
+        RTE_TRY(mk_second(h, u_minus, nrhs, true));
+        RTE_CUDA_TRY(cudaGetLastError());
+        return tc_gemm_error(s);
+    }
     apply_A(s, d, u_plus, h->z1, nrhs);                                   // z1 = A u^+
     axpby_per_rhs(s, l_minus, h->z1, len, nrhs, nullptr, 1.0, nullptr, -1.0);   // l^- - z1
     RTE_TRY(mk_inv(h, h->z1, h->z2, nrhs));
@@ -2228,11 +2316,7 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
     double worst = 0.0, energy = 0.0;
     for (it = 0;; ++it) {
         // r = (E - K^+) u - q   (Algorithm 3: residual)
-        RTE_TRY(apply_E(h, u, r, nrhs, true));
-        {
-            Scope scp(h, "axpy");
-            axpby_per_rhs(s, q, r, len, nrhs, nullptr, -1.0, nullptr, 1.0);
-        }
+        RTE_TRY(apply_E(h, u, r, nrhs, true, q));
         dot_per_rhs(s, r, r, len, nrhs, h->partial, sc);
         if (it > 0) {
             // ||u_n - u_{n-1}||^2_{E-K} = delta^T (r_n - r_{n-1})

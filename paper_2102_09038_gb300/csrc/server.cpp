@@ -237,7 +237,8 @@ size_t rte_estimate_bytes(const rte_problem* p, const rte_options* o, int nrhs) 
     const bool p1_pcg = o && (o->p1_route == RTE_P1_PCG ||
                               (o->p1_route == RTE_P1_AUTO && o->precision != RTE_FP64));
     if (p1_pcg) b += r * nRp * nSp * 8 * 2;    // the P_1 PCG's r and p
-    b += nSm * nSm * 8 * 5 + nSp * nSp * 8 * 3;   // dense angular factors, slices
+    // dense angular factors (V, W and their transposes, S) and slices
+    b += nSm * nSm * 8 * 9 + nSp * nSp * 8 * 3;
     const bool split = o && (o->dgemm == RTE_DGEMM_SPLIT ||
                              (o->dgemm == RTE_DGEMM_AUTO && o->precision != RTE_FP64));
     if (split && o->mk_route != RTE_MK_PCG)
