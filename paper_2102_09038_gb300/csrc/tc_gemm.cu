@@ -7,12 +7,18 @@
 //   second operand given K-major as Bt[N x K] (K contiguous)
 //
 // Operands are BF16 (tcgen05.mma kind::f16) or FP32 read as TF32
-// (kind::tf32); accumulation is FP32 in tensor memory.  One CTA computes one
-// 128 x BN tile: warp 0 lane 0 issues TMA loads into a 4-stage shared-memory
-// ring (128-byte swizzle), warp 1 lane 0 issues the MMAs, and all four warps
-// then drain the accumulator with tcgen05.ld and apply the epilogue.  Every
-// wait on an mbarrier is bounded: on timeout the kernel records an error flag
-// and leaves instead of hanging.
+// (kind::tf32); accumulation is FP32 in tensor memory.  Tiles of 128 x BN:
+// warp 0 issues TMA loads into a 4-stage shared-memory ring (128-byte
+// swizzle), warp 1 the MMAs, warps 2 to 9 drain the accumulators with
+// tcgen05.ld and apply the epilogue.  Blocks are persistent and the
+// accumulator is double-buffered, so the loads and MMAs of a tile run under
+// the epilogue of the one before: at the solver's sizes (K = 768) a
+// tile's epilogue (a division per element, 64 to 128 KB of stores) takes about
+// as long as its MMAs, and one tile per block exposed both.  Measured in a
+// solve, 32768 x 768 x 768 BF16: with the shifted inverse in the epilogue 152
+// -> 79 us, the plain product to FP32 81 -> 57 us.  Every wait on an mbarrier
+// is bounded: on timeout the kernel records an error flag and leaves instead
+// of hanging.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -38,134 +44,181 @@ using namespace tc;
 constexpr int kBM = 128;
 constexpr int kStages = 4;
 
+constexpr int kEpiWarps = 8;
+constexpr int kTcThreads = 64 + 32 * kEpiWarps;
+
 template <int BN, bool TF32, typename TOut>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
 k_tc_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
           int M, int N, int K, TOut* __restrict__ C, int ldc, int epi,
           const float* __restrict__ at, const float* __restrict__ as,
           const float* __restrict__ lam, int rows, float beta) {
     constexpr uint32_t kABytes = kBM * kRowBytes;
     constexpr uint32_t kBBytes = BN * kRowBytes;
-    constexpr uint32_t kTmemCols = BN;   // FP32 accumulator: one column per N
+    constexpr uint32_t kTmemCols = 2 * BN;   // two FP32 accumulators, one column per N
+    constexpr int kKB = TF32 ? 32 : 64;      // values of K per stage
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // 1024-byte alignment of the operand ring (swizzle atoms)
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sA = smem;
     uint8_t* sB = smem + kStages * kABytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + kStages * kBBytes);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 1);
+    __shared__ __align__(8) uint64_t bars[2 * kStages + 4];
+    __shared__ uint32_t tmem_slot;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * BN;
-    const int kblocks = (K + (TF32 ? 32 : 64) - 1) / (TF32 ? 32 : 64);
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kStages),
-                   done = smem_u32(bars + 2 * kStages);
+    const int ntn = (N + BN - 1) / BN, tiles = ntn * ((M + kBM - 1) / kBM);
+    const int kblocks = (K + kKB - 1) / kKB;
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kStages,
+                   accf0 = full0 + 16 * kStages, acce0 = accf0 + 16;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(full0 + 8 * s, 1);
             mbar_init(empty0 + 8 * s, 1);
         }
-        mbar_init(done, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(accf0 + 8 * b, 1);
+            mbar_init(acce0 + 8 * b, kEpiWarps);   // one arrival per epilogue warp
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(tmem_slot)),
+                         smem_u32(&tmem_slot)),
                      "r"(kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = tmem_slot;
     bool ok = true;
 
     if (warp == 0 && lane == 0) {
         // ------------------------------------------------ TMA producer
-        for (int kb = 0; kb < kblocks && ok; ++kb) {
-            const int s = kb % kStages;
-            const uint32_t ph = (kb / kStages) & 1;
-            if (!mbar_wait(empty0 + 8 * s, ph ^ 1)) { ok = false; break; }
-            mbar_expect_tx(full0 + 8 * s, kABytes + kBBytes);
-            const int kx = kb * (TF32 ? 32 : 64);
-            tma_load_2d(smem_u32(sA + s * kABytes), &mapA, full0 + 8 * s, kx, m0);
-            tma_load_2d(smem_u32(sB + s * kBBytes), &mapB, full0 + 8 * s, kx, n0);
-        }
-    } else if (warp == 1 && lane == 0) {
-        // ------------------------------------------------- MMA issuer
-        uint32_t idesc = (1u << 4)                                   // D: FP32
-                         | ((TF32 ? 2u : 1u) << 7)                   // A: TF32 / BF16
-                         | ((TF32 ? 2u : 1u) << 10)                  // B: TF32 / BF16
-                         | ((uint32_t)(BN >> 3) << 17)               // N
-                         | ((uint32_t)(kBM >> 4) << 24);             // M
-        for (int kb = 0; kb < kblocks && ok; ++kb) {
-            const int s = kb % kStages;
-            const uint32_t ph = (kb / kStages) & 1;
-            if (!mbar_wait(full0 + 8 * s, ph)) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_u32(sA + s * kABytes), b0 = smem_u32(sB + s * kBBytes);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {   // 4 MMAs of 32 bytes of K each
-                mma_issue(TF32, tmem, sw128_desc(a0 + 32 * kk), sw128_desc(b0 + 32 * kk), idesc,
-                          (kb > 0 || kk > 0) ? 1u : 0u);
+        int st = 0;
+        uint32_t ph = 1, loaded = 0;
+        for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
+            const int m0 = tile / ntn * kBM, n0 = tile % ntn * BN;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (!mbar_wait(empty0 + 8 * st, ph)) { ok = false; break; }
+                mbar_expect_tx(full0 + 8 * st, kABytes + kBBytes);
+                tma_load_2d(smem_u32(sA + st * kABytes), &mapA, full0 + 8 * st, kb * kKB, m0);
+                tma_load_2d(smem_u32(sB + st * kBBytes), &mapB, full0 + 8 * st, kb * kKB, n0);
+                loaded |= 1u << st;
+                if (++st == kStages) { st = 0; ph ^= 1; }
             }
-            mma_commit(empty0 + 8 * s);   // frees the stage once these MMAs have read it
         }
-        mma_commit(done);
+        // after a timeout: the copies still in flight land before the block
+        // leaves (stages before st hold one of this round)
+        if (!ok)
+            for (int i = 0; i < kStages; ++i)
+                if (loaded >> i & 1u) mbar_wait(full0 + 8 * i, i < st ? ph ^ 1u : ph);
+    } else if (warp == 1) {
+        // ------------------------------------------------- MMA issuer
+        // the whole warp keeps warp-uniform values; one lane issues
+        constexpr uint32_t idesc = (1u << 4)                                   // D: FP32
+                                   | ((TF32 ? 2u : 1u) << 7)                   // A: TF32 / BF16
+                                   | ((TF32 ? 2u : 1u) << 10)                  // B: TF32 / BF16
+                                   | ((uint32_t)(BN >> 3) << 17)               // N
+                                   | ((uint32_t)(kBM >> 4) << 24);             // M
+        const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        int st = 0;
+        uint32_t ph = 0, used = 0;
+        for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++used) {
+            const uint32_t buf = used & 1u;
+            if (!mbar_wait_warp(acce0 + 8 * buf, (used >> 1 & 1u) ^ 1u)) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t d = tm + buf * BN;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (!mbar_wait_warp(full0 + 8 * st, ph)) { ok = false; break; }
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t da = da0 + (uint64_t)(st * (kABytes >> 4)),
+                               db = db0 + (uint64_t)(st * (kBBytes >> 4));
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)   // 4 MMAs of 32 bytes of K each
+                        mma_issue(TF32, d, da + 2 * kk, db + 2 * kk, idesc,
+                                  (kb > 0 || kk > 0) ? 1u : 0u);
+                    mma_commit(empty0 + 8 * st);   // frees the stage once these MMAs have read it
+                }
+                if (++st == kStages) { st = 0; ph ^= 1; }
+            }
+            if (ok && elect_one()) mma_commit(accf0 + 8 * buf);
+        }
+    } else if (warp >= 2) {
+        // ---------------------------------------------------------- epilogue
+        const int wq = warp & 3, half = (warp - 2) >> 2;
+        uint32_t used = 0;
+        for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++used) {
+            const uint32_t buf = used & 1u;
+            const int m0 = tile / ntn * kBM, n0 = tile % ntn * BN;
+            const int row = m0 + wq * 32 + lane;
+            float fat = 0.f, fas = 0.f;
+            if (epi != 0 && row < M) {
+                const int rr = row % rows;
+                fat = at[rr];
+                fas = as[rr];
+            }
+            if (ok) {
+                int got = 1;
+                if (lane == 0) got = mbar_wait(accf0 + 8 * buf, used >> 1 & 1u);
+                ok = __shfl_sync(0xffffffffu, got, 0) != 0;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int c0 = half * (BN / 2); c0 < (half + 1) * (BN / 2); c0 += 16) {
+                float v[16];
+                // every lane of the warp takes part in the load, whatever its row
+                tmem_ld16(tmem + ((uint32_t)(wq * 32) << 16) + buf * BN + (uint32_t)c0, v);
+                if (c0 + 16 == (half + 1) * (BN / 2)) {
+                    // the buffer is free once every warp has read its part
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(acce0 + 8 * buf);
+                }
+                if (!ok || row >= M || n0 + c0 >= N) continue;
+                TOut* dst = C + (size_t)row * ldc + n0 + c0;
+                const bool full = n0 + c0 + 16 <= N && beta == 0.f &&
+                                  ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
+                if (full) {
+                    if (epi == 1) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            v[i] = v[i] / (fat - __ldg(lam + n0 + c0 + i) * fas);
+                    }
+                    if constexpr (sizeof(TOut) == 4) {
+                        float4* d4 = reinterpret_cast<float4*>(dst);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            d4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    } else {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+                            w[i] = *reinterpret_cast<uint32_t*>(&h);
+                        }
+                        uint4* d4 = reinterpret_cast<uint4*>(dst);
+                        d4[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                        d4[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    }
+                    continue;
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int col = n0 + c0 + i;
+                    if (col >= N) break;
+                    float x = v[i];
+                    if (epi == 1) x = x / (fat - lam[col] * fas);
+                    if (beta != 0.f) x += beta * static_cast<float>(dst[i]);
+                    dst[i] = static_cast<TOut>(x);
+                }
+            }
+        }
     }
     __syncwarp();
-    // ---------------------------------------------------------- epilogue
-    ok = mbar_wait(done, 0);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int row = m0 + warp * 32 + lane;
-    float fat = 0.f, fas = 0.f;
-    if (epi != 0 && row < M) {
-        const int rr = row % rows;
-        fat = at[rr];
-        fas = as[rr];
-    }
-    for (int c0 = 0; c0 < BN; c0 += 16) {
-        float v[16];
-        // every lane of the warp takes part in the load, whatever its row
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
-        if (!ok || row >= M) continue;
-        TOut* dst = C + (size_t)row * ldc + n0 + c0;
-        const bool full = n0 + c0 + 16 <= N && beta == 0.f &&
-                          ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
-        if (full) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (epi == 1) v[i] = v[i] / (fat - lam[n0 + c0 + i] * fas);
-            if constexpr (sizeof(TOut) == 4) {
-                float4* d4 = reinterpret_cast<float4*>(dst);
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    d4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-            } else {
-                uint32_t w[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-                    w[i] = *reinterpret_cast<uint32_t*>(&h);
-                }
-                uint4* d4 = reinterpret_cast<uint4*>(dst);
-                d4[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                d4[1] = make_uint4(w[4], w[5], w[6], w[7]);
-            }
-            continue;
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int col = n0 + c0 + i;
-            if (col >= N) break;
-            float x = v[i];
-            if (epi == 1) x = x / (fat - lam[col] * fas);
-            if (beta != 0.f) x += beta * static_cast<float>(dst[i]);
-            dst[i] = static_cast<TOut>(x);
-        }
-    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -175,7 +228,7 @@ k_tc_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
 
 template <int BN>
 constexpr size_t smem_bytes() {
-    return 1024 + (size_t)kStages * (kBM + BN) * kRowBytes + (2 * kStages + 1) * 8 + 16;
+    return 1024 + (size_t)kStages * (kBM + BN) * kRowBytes;   // 1024: alignment
 }
 
 template <int BN, bool TF32, typename TOut>
@@ -187,10 +240,11 @@ int launch(cudaStream_t s, const TcGemmArgs& g) {
     const size_t sm = smem_bytes<BN>();
     // set on every call: the attribute is per device, and cheap to set
     RTE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    dim3 grid((g.N + BN - 1) / BN, (g.M + kBM - 1) / kBM);
+    const long long tiles = (long long)((g.N + BN - 1) / BN) * ((g.M + kBM - 1) / kBM);
     count_launches(1);
-    kern<<<grid, 128, sm, s>>>(ma, mb, g.M, g.N, g.K, static_cast<TOut*>(g.C), g.ldc, g.epi,
-                               g.at, g.as, g.lam, g.rows, g.beta);
+    kern<<<(unsigned)std::min<long long>(tiles, device_sm_count()), kTcThreads, sm, s>>>(
+        ma, mb, g.M, g.N, g.K, static_cast<TOut*>(g.C), g.ldc, g.epi, g.at, g.as, g.lam, g.rows,
+        g.beta);
     RTE_CUDA_TRY(cudaGetLastError());
     return RTE_OK;
 }
@@ -300,10 +354,6 @@ __host__ __device__ constexpr int oz_run(int S, int BN, int a, int b) {
     while (a + b + len < S && oz_group(a, b + len) == oz_group(a, b) + len && (len + 1) * BN <= 256)
         ++len;
     return len;
-}
-
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar,

@@ -39,6 +39,10 @@ static __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t byt
                  : "memory");
 }
 
+static __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
 static __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
