@@ -161,10 +161,34 @@ void convert(cudaStream_t s, const double* x, float* y, size_t n);
 // x = beta x + uc W^T, one warp per row, for dP <= 16 (false otherwise: the
 // caller falls back to the general GEMM); W, WT in FP64 or FP32 (products and
 // sums in that type, FP64 vectors at the interface).
+// sub: restrict x - sub.  U, D, status: leave x and update U -= result, D =
+// -result unless the coarse solve gave up.
 bool restrict_rows(cudaStream_t s, int rows, int nSp, int dP, const double* x, const double* W,
-                   const float* W32, double* qc);
+                   const float* W32, double* qc, const float* sub = nullptr);
 bool prolong_rows(cudaStream_t s, int rows, int nSp, int dP, const double* uc, const double* WT,
-                  const float* WT32, double* x, double beta);
+                  const float* WT32, double* x, double beta, double* U = nullptr,
+                  double* D = nullptr, const SolveStatus* status = nullptr);
+
+// Vector passes of the mixed modes' P_1 steps and of the outer iteration
+// (kernels.cu); len values per right-hand side, an even number; partial holds
+// 3 nrhs 1024 doubles.
+// P = Y, F = (float)Y, rho = R.Y
+void p1_start(cudaStream_t s, const double* R, const double* Y, double* P, float* F, size_t len,
+              int nrhs, double* partial, double* rho);
+// alpha = rho / P.F2
+void p1_length(cudaStream_t s, const double* P, const float* F2, size_t len, int nrhs,
+               double* partial, double* rho, double* alpha);
+// Z = alpha P (first) or Z += alpha P; R = B - alpha F2, or (last) F = (float)Z
+void p1_step(cudaStream_t s, const double* alpha, bool first, bool last, const double* P,
+             const float* F2, const double* B, double* Z, double* R, float* F, size_t len, int nrhs);
+// beta = R.Y / rho, rho = R.Y, P = Y + beta P, F = (float)P
+void p1_direction(cudaStream_t s, const double* R, const double* Y, double* P, float* F, size_t len,
+                  int nrhs, double* partial, double* rho, double* beta);
+// out = [R.R] and, with D, [D.R], [D.Rp], nrhs values each
+void residual_sums(cudaStream_t s, const double* R, const double* D, const double* Rp, size_t len,
+                   int nrhs, double* partial, double* out);
+// U -= S, D = -S
+void update_solution(cudaStream_t s, const double* S, double* U, double* D, size_t n);
 void convert(cudaStream_t s, const float* x, double* y, size_t n);
 void convert(cudaStream_t s, const float* x, __nv_bfloat16* y, size_t n);
 void convert(cudaStream_t s, const double* x, __nv_bfloat16* y, size_t n);
@@ -223,6 +247,10 @@ int e0_direct_solve(cudaStream_t s, const DevSystem& d, const double* B, double*
                     bool fp64);
 // Reads and clears the flag a timed-out factor-block wait sets (synchronises s).
 int e0_direct_error(cudaStream_t s);
+// The same in two halves around a synchronisation of the caller's: the copy
+// of the flag to (pinned) host memory, and its check afterwards.
+int e0_direct_error_fetch(cudaStream_t s, int* host);
+int e0_direct_error_check(cudaStream_t s, int flag);
 // Limit of one such wait on the current device (SM clock cycles).
 int e0_set_wait_cycles(long long cycles);
 

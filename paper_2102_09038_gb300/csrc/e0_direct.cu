@@ -669,17 +669,23 @@ int e0_direct_solve(cudaStream_t s, const DevSystem& d, const double* B, double*
     return solve<float>(s, d, d.e0lu32, B, X, nrhs);
 }
 
+int e0_direct_error_fetch(cudaStream_t s, int* host) {
+    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(host, g_e0_error, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
+    return RTE_OK;
+}
+
+int e0_direct_error_check(cudaStream_t s, int flag) {
+    if (!flag) return RTE_OK;
+    const int zero = 0;
+    cudaMemcpyToSymbolAsync(g_e0_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
+    return fail(RTE_ERR_TIMEOUT, "a wait for a staged E_0 factor record timed out");
+}
+
 int e0_direct_error(cudaStream_t s) {
     int e = 0;
-    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(&e, g_e0_error, sizeof(int), 0, cudaMemcpyDeviceToHost,
-                                           s));
+    RTE_TRY(e0_direct_error_fetch(s, &e));
     RTE_CUDA_TRY(cudaStreamSynchronize(s));
-    if (e) {
-        const int zero = 0;
-        cudaMemcpyToSymbolAsync(g_e0_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-        return fail(RTE_ERR_TIMEOUT, "a wait for a staged E_0 factor record timed out");
-    }
-    return RTE_OK;
+    return e0_direct_error_check(s, e);
 }
 
 int e0_set_wait_cycles(long long cycles) {

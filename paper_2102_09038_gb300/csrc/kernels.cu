@@ -803,6 +803,175 @@ k_even_lo(int m, int nSp, int nrhs, const float* __restrict__ cell_D, const floa
     *reinterpret_cast<P4*>(Y + (size_t)ri * nSp + k) = out;
 }
 
+// ------------------------------------ vector passes of the mixed iteration
+// The P_1 steps and the update of the outer iteration as few passes over the
+// vectors: each kernel below reads what it needs once and writes every form
+// (FP64, and the FP32 copy the inner operator takes) of its result, and sums
+// what is needed of it; the separate copies, conversions, axpys and dots took
+// 45 array passes and 30 launches an iteration more.  Bound by memory, and on
+// small meshes by the launches.  Measured, whole solve with the iteration's
+// one synchronisation in place of two: 128 x 128 / 512 triangles 76.2 -> 71.2
+// ms, 77 x 77 with three right-hand sides 51.5 -> 41.9, 32 x 32 / 128
+// triangles 3.5 -> 2.9.  W as above; one right-hand side per blockIdx.y, len
+// values each.
+
+// per-block sums of NS products into partial[(q nrhs + r) 1024 + block]
+template <int NS>
+__device__ void store_partials(double (&s)[NS], double* __restrict__ partial) {
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        const double v = block_sum<256>(s[q]);
+        if (threadIdx.x == 0)
+            partial[((size_t)q * gridDim.y + blockIdx.y) * 1024 + blockIdx.x] = v;
+    }
+}
+
+// P = Y, F = Y in FP32, partial sums of R.Y
+template <int W>
+__global__ void __launch_bounds__(256)
+k_p1_start(const double* __restrict__ R, const double* __restrict__ Y, double* __restrict__ P,
+           float* __restrict__ F, size_t len, double* __restrict__ partial) {
+    const size_t o = (size_t)blockIdx.y * len;
+    double s[1] = {0.0};
+    for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * W; e < len; e += (size_t)gridDim.x * 256 * W) {
+        const Pack<double, W> r = *reinterpret_cast<const Pack<double, W>*>(R + o + e);
+        const Pack<double, W> y = *reinterpret_cast<const Pack<double, W>*>(Y + o + e);
+        Pack<float, W> f;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            f.v[w] = (float)y.v[w];
+            s[0] = fma(r.v[w], y.v[w], s[0]);
+        }
+        *reinterpret_cast<Pack<double, W>*>(P + o + e) = y;
+        *reinterpret_cast<Pack<float, W>*>(F + o + e) = f;
+    }
+    store_partials<1>(s, partial);
+}
+
+// partial sums of P.F2 (F2 the FP32 result of an inner apply)
+__global__ void __launch_bounds__(256)
+k_p1_dot(const double* __restrict__ P, const float* __restrict__ F2, size_t len,
+         double* __restrict__ partial) {
+    const size_t o = (size_t)blockIdx.y * len;
+    double s[1] = {0.0};
+    for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * 2; e < len; e += (size_t)gridDim.x * 512) {
+        const double2 p = *reinterpret_cast<const double2*>(P + o + e);
+        const float2 f = *reinterpret_cast<const float2*>(F2 + o + e);
+        s[0] = fma(p.x, (double)f.x, s[0]);
+        s[0] = fma(p.y, (double)f.y, s[0]);
+    }
+    store_partials<1>(s, partial);
+}
+
+// One P_1 step: Z = alpha P (first) or Z += alpha P; R = B - alpha F2 unless
+// it is the last one (B: the right-hand side on the first step, R itself
+// after), which leaves F = Z in FP32 instead.
+template <int W>
+__global__ void __launch_bounds__(256)
+k_p1_step(const double* __restrict__ alpha, int first, int last, const double* __restrict__ P,
+          const float* __restrict__ F2, const double* B, double* Z, double* R,
+          float* __restrict__ F, size_t len) {
+    const size_t o = (size_t)blockIdx.y * len;
+    const double a = alpha[blockIdx.y];
+    for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * W; e < len; e += (size_t)gridDim.x * 256 * W) {
+        const Pack<double, W> p = *reinterpret_cast<const Pack<double, W>*>(P + o + e);
+        Pack<double, W> z;
+        if (!first) z = *reinterpret_cast<const Pack<double, W>*>(Z + o + e);
+#pragma unroll
+        for (int w = 0; w < W; ++w) z.v[w] = first ? a * p.v[w] : a * p.v[w] + z.v[w];
+        *reinterpret_cast<Pack<double, W>*>(Z + o + e) = z;
+        if (last) {
+            Pack<float, W> f;
+#pragma unroll
+            for (int w = 0; w < W; ++w) f.v[w] = (float)z.v[w];
+            *reinterpret_cast<Pack<float, W>*>(F + o + e) = f;
+        } else {
+            Pack<double, W> b = *reinterpret_cast<const Pack<double, W>*>(B + o + e);
+            const Pack<float, W> g = *reinterpret_cast<const Pack<float, W>*>(F2 + o + e);
+#pragma unroll
+            for (int w = 0; w < W; ++w) b.v[w] = -a * (double)g.v[w] + b.v[w];
+            *reinterpret_cast<Pack<double, W>*>(R + o + e) = b;
+        }
+    }
+}
+
+// P = Y + beta P, F = P in FP32
+__global__ void __launch_bounds__(256)
+k_p1_direction(const double* __restrict__ beta, const double* __restrict__ Y, double* __restrict__ P,
+               float* __restrict__ F, size_t len) {
+    const size_t o = (size_t)blockIdx.y * len;
+    const double b = beta[blockIdx.y];
+    for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * 2; e < len; e += (size_t)gridDim.x * 512) {
+        const double2 y = *reinterpret_cast<const double2*>(Y + o + e);
+        double2 p = *reinterpret_cast<const double2*>(P + o + e);
+        p.x = y.x + b * p.x;
+        p.y = y.y + b * p.y;
+        *reinterpret_cast<double2*>(P + o + e) = p;
+        *reinterpret_cast<float2*>(F + o + e) = make_float2((float)p.x, (float)p.y);
+    }
+}
+
+// Sum of a right-hand side's partials, and the scalar it gives: op 0: out =
+// sum; 1: out = rho / sum (a step length); 2: out = sum / rho and rho = sum (a
+// direction's factor).  blockIdx.x: sum q nrhs + r.
+__global__ void __launch_bounds__(256)
+k_sum_scalar(const double* __restrict__ partial, int nb, int op, double* rho,
+             double* __restrict__ out) {
+    const int r = blockIdx.x;
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 256) s += partial[(size_t)r * 1024 + b];
+    s = block_sum<256>(s);
+    if (threadIdx.x != 0) return;
+    if (op == 0) {
+        out[r] = s;
+    } else if (op == 1) {
+        out[r] = s != 0.0 ? rho[r] / s : 0.0;
+    } else {
+        out[r] = rho[r] != 0.0 ? s / rho[r] : 0.0;
+        rho[r] = s;
+    }
+}
+
+// partial sums of R.R and, with D, D.R and D.Rp
+template <bool ALL>
+__global__ void __launch_bounds__(256)
+k_residual_sums(const double* __restrict__ R, const double* __restrict__ D,
+                const double* __restrict__ Rp, size_t len, double* __restrict__ partial) {
+    const size_t o = (size_t)blockIdx.y * len;
+    double s[ALL ? 3 : 1] = {};
+    for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * 2; e < len; e += (size_t)gridDim.x * 512) {
+        const double2 r = *reinterpret_cast<const double2*>(R + o + e);
+        s[0] = fma(r.x, r.x, s[0]);
+        s[0] = fma(r.y, r.y, s[0]);
+        if constexpr (ALL) {
+            const double2 d = *reinterpret_cast<const double2*>(D + o + e);
+            const double2 p = *reinterpret_cast<const double2*>(Rp + o + e);
+            s[1] = fma(d.x, r.x, s[1]);
+            s[1] = fma(d.y, r.y, s[1]);
+            s[2] = fma(d.x, p.x, s[2]);
+            s[2] = fma(d.y, p.y, s[2]);
+        }
+    }
+    store_partials<ALL ? 3 : 1>(s, partial);
+}
+
+// U -= S, D = -S
+template <int W>
+__global__ void __launch_bounds__(256)
+k_update(const double* __restrict__ S, double* __restrict__ U, double* __restrict__ D, size_t n) {
+    for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * W; e < n; e += (size_t)gridDim.x * 256 * W) {
+        const Pack<double, W> v = *reinterpret_cast<const Pack<double, W>*>(S + e);
+        Pack<double, W> u = *reinterpret_cast<const Pack<double, W>*>(U + e), d;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            u.v[w] -= v.v[w];
+            d.v[w] = -v.v[w];
+        }
+        *reinterpret_cast<Pack<double, W>*>(U + e) = u;
+        *reinterpret_cast<Pack<double, W>*>(D + e) = d;
+    }
+}
+
 // whether pointers allow W = 2 accesses of T (null ones do)
 template <typename T, typename... Ps>
 bool paired(const Ps*... p) {
@@ -961,6 +1130,65 @@ void axpby_per_rhs(cudaStream_t s, const float* x, float* y, size_t len, int nrh
     k_axpby<float><<<grid_for(len * nrhs), kThreads, 0, s>>>(x, y, len, nrhs, a, ca, b, cb);
 }
 
+// blocks of a vector pass over len values, and of its partial sums (<= 1024)
+static int pass_blocks(size_t len) {
+    return (int)std::min<size_t>(1024, std::max<size_t>(1, (len + 2047) / 2048));
+}
+
+void p1_start(cudaStream_t s, const double* R, const double* Y, double* P, float* F, size_t len,
+              int nrhs, double* partial, double* rho) {
+    const int nb = pass_blocks(len);
+    count_launches(2);
+    if (paired<double>(R))
+        k_p1_start<2><<<dim3(nb, nrhs), 256, 0, s>>>(R, Y, P, F, len, partial);
+    else
+        k_p1_start<1><<<dim3(nb, nrhs), 256, 0, s>>>(R, Y, P, F, len, partial);
+    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 0, nullptr, rho);
+}
+
+void p1_length(cudaStream_t s, const double* P, const float* F2, size_t len, int nrhs,
+               double* partial, double* rho, double* alpha) {
+    const int nb = pass_blocks(len);
+    count_launches(2);
+    k_p1_dot<<<dim3(nb, nrhs), 256, 0, s>>>(P, F2, len, partial);
+    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 1, rho, alpha);
+}
+
+void p1_step(cudaStream_t s, const double* alpha, bool first, bool last, const double* P,
+             const float* F2, const double* B, double* Z, double* R, float* F, size_t len, int nrhs) {
+    const int nb = pass_blocks(len);
+    count_launches(1);
+    if (paired<double>(B, Z))
+        k_p1_step<2><<<dim3(nb, nrhs), 256, 0, s>>>(alpha, first, last, P, F2, B, Z, R, F, len);
+    else
+        k_p1_step<1><<<dim3(nb, nrhs), 256, 0, s>>>(alpha, first, last, P, F2, B, Z, R, F, len);
+}
+
+void p1_direction(cudaStream_t s, const double* R, const double* Y, double* P, float* F, size_t len,
+                  int nrhs, double* partial, double* rho, double* beta) {
+    const int nb = pass_blocks(len);
+    count_launches(3);
+    k_dot_partial<double><<<dim3(nb, nrhs), 256, 0, s>>>(R, Y, len, partial);
+    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 2, rho, beta);
+    k_p1_direction<<<dim3(nb, nrhs), 256, 0, s>>>(beta, Y, P, F, len);
+}
+
+void residual_sums(cudaStream_t s, const double* R, const double* D, const double* Rp, size_t len,
+                   int nrhs, double* partial, double* out) {
+    const int nb = pass_blocks(len);
+    count_launches(2);
+    if (D) k_residual_sums<true><<<dim3(nb, nrhs), 256, 0, s>>>(R, D, Rp, len, partial);
+    else k_residual_sums<false><<<dim3(nb, nrhs), 256, 0, s>>>(R, D, Rp, len, partial);
+    k_sum_scalar<<<(D ? 3 : 1) * nrhs, 256, 0, s>>>(partial, nb, 0, nullptr, out);
+}
+
+void update_solution(cudaStream_t s, const double* S, double* U, double* D, size_t n) {
+    const unsigned blocks = (unsigned)std::min<size_t>((n + 511) / 512, 65535);
+    count_launches(1);
+    if (paired<double>(U)) k_update<2><<<blocks, 256, 0, s>>>(S, U, D, n);
+    else k_update<1><<<blocks, 256, 0, s>>>(S, U, D, n);
+}
+
 void fill_uniform(cudaStream_t s, double* x, size_t n, unsigned long long seed) {
     count_launches(1);
     k_fill_uniform<<<grid_for(n), kThreads, 0, s>>>(x, n, seed);
@@ -971,8 +1199,10 @@ void fill_uniform(cudaStream_t s, double* x, size_t n, unsigned long long seed) 
 // qc[row][j] = sum_k x[row][k] W[k][j], one warp per row: lanes stride over
 // k with 16 partial sums each, reduced across the warp by halving exchanges
 // (31 shuffles leave lane j holding the sum of column j mod 16).
+// sub set: of x - sub instead.
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(int rows, int nSp, int dP, const double* __restrict__ x,
+                                                  const float* __restrict__ sub,
                                                   const T* __restrict__ W, double* __restrict__ qc) {
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (row >= rows) return;
@@ -981,7 +1211,7 @@ __global__ void __launch_bounds__(256) k_restrict(int rows, int nSp, int dP, con
     for (int j = 0; j < 16; ++j) v[j] = T(0);
     const double* xr = x + (size_t)row * nSp;
     for (int k = lane; k < nSp; k += 32) {
-        const T xv = (T)__ldg(xr + k);
+        const T xv = (T)(sub ? __ldg(xr + k) - (double)__ldg(sub + (size_t)row * nSp + k) : __ldg(xr + k));
         const T* w = W + (size_t)k * dP;
 #pragma unroll
         for (int j = 0; j < 16; ++j)
@@ -1003,10 +1233,15 @@ __global__ void __launch_bounds__(256) k_restrict(int rows, int nSp, int dP, con
 }
 
 // x[row][k] = beta x[row][k] + sum_j uc[row][j] WT[j][k], one warp per row.
+// U set (the outer update): x stays, U -= that and D = -that, unless the
+// coarse solve's status says that it gave up.
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong(int rows, int nSp, int dP, const double* __restrict__ uc,
                                                  const T* __restrict__ WT, double* __restrict__ x,
-                                                 double beta) {
+                                                 double beta, double* __restrict__ U,
+                                                 double* __restrict__ D,
+                                                 const SolveStatus* __restrict__ status) {
+    if (U && status->timed_out) return;
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (row >= rows) return;
     const T mine = lane < dP ? (T)uc[(size_t)row * dP + lane] : T(0);
@@ -1019,31 +1254,38 @@ __global__ void __launch_bounds__(256) k_prolong(int rows, int nSp, int dP, cons
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             if (j < dP) acc = fma(u[j], __ldg(WT + (size_t)j * nSp + k), acc);
-        xr[k] = beta == 0.0 ? (double)acc : beta * xr[k] + (double)acc;
+        const double v = beta == 0.0 ? (double)acc : beta * xr[k] + (double)acc;
+        if (U) {
+            U[(size_t)row * nSp + k] -= v;
+            D[(size_t)row * nSp + k] = -v;
+        } else {
+            xr[k] = v;
+        }
     }
 }
 
 bool restrict_rows(cudaStream_t s, int rows, int nSp, int dP, const double* x, const double* W,
-                   const float* W32, double* qc) {
+                   const float* W32, double* qc, const float* sub) {
     if (dP < 1 || dP > 16 || rows <= 0) return false;
     const unsigned blocks = (unsigned)(((size_t)rows * 32 + 255) / 256);
     count_launches(1);
     if (W32)
-        k_restrict<float><<<blocks, 256, 0, s>>>(rows, nSp, dP, x, W32, qc);
+        k_restrict<float><<<blocks, 256, 0, s>>>(rows, nSp, dP, x, sub, W32, qc);
     else
-        k_restrict<double><<<blocks, 256, 0, s>>>(rows, nSp, dP, x, W, qc);
+        k_restrict<double><<<blocks, 256, 0, s>>>(rows, nSp, dP, x, sub, W, qc);
     return true;
 }
 
 bool prolong_rows(cudaStream_t s, int rows, int nSp, int dP, const double* uc, const double* WT,
-                  const float* WT32, double* x, double beta) {
+                  const float* WT32, double* x, double beta, double* U, double* D,
+                  const SolveStatus* status) {
     if (dP < 1 || dP > 16 || rows <= 0) return false;
     const unsigned blocks = (unsigned)(((size_t)rows * 32 + 255) / 256);
     count_launches(1);
     if (WT32)
-        k_prolong<float><<<blocks, 256, 0, s>>>(rows, nSp, dP, uc, WT32, x, beta);
+        k_prolong<float><<<blocks, 256, 0, s>>>(rows, nSp, dP, uc, WT32, x, beta, U, D, status);
     else
-        k_prolong<double><<<blocks, 256, 0, s>>>(rows, nSp, dP, uc, WT, x, beta);
+        k_prolong<double><<<blocks, 256, 0, s>>>(rows, nSp, dP, uc, WT, x, beta, U, D, status);
     return true;
 }
 

@@ -69,6 +69,11 @@ struct rte_handle {
     void *zl1 = nullptr, *zl2 = nullptr, *xl = nullptr;
     float* zf = nullptr;
     double *partial = nullptr, *sc = nullptr;                               // reductions
+    // pinned host memory of the outer iteration's one synchronisation: the
+    // residual sums, the coarse solve's status, the E_0 sweeps' flag
+    double* host_sums = nullptr;
+    SolveStatus* host_status = nullptr;
+    int* host_e0_error = nullptr;
     void* e0work = nullptr;
     size_t e0bytes = 0;
     void* cowork = nullptr;
@@ -892,7 +897,14 @@ int alloc_workspace(rte_handle* h, int nrhs) {
     }
     RTE_TRY(dalloc(h, &h->c1, nc));
     RTE_TRY(dalloc(h, &h->c2, nc));
-    RTE_TRY(dalloc(h, &h->partial, (size_t)nrhs * 1024));
+    RTE_TRY(dalloc(h, &h->partial, (size_t)nrhs * 3 * 1024));
+    char* pin = nullptr;
+    if (cudaMallocHost(&pin, (size_t)nrhs * 3 * sizeof(double) + sizeof(SolveStatus) + sizeof(int)) != cudaSuccess)
+        return fail(RTE_ERR_NOMEM, "pinned iteration state");
+    h->host_sums = reinterpret_cast<double*>(pin);
+    h->host_status = reinterpret_cast<SolveStatus*>(h->host_sums + (size_t)nrhs * 3);
+    h->host_e0_error = reinterpret_cast<int*>(h->host_status + 1);
+    *h->host_e0_error = 0;
     RTE_TRY(dalloc(h, &h->sc, (size_t)nrhs * 16));
     char* w = nullptr;
     if (!d.e0_direct) {
@@ -1366,15 +1378,18 @@ int e0_inv(rte_handle* h, const double* b, double* x, int nrhs) {
 // products in FP32
 constexpr double kCoarseF32Tol = 1e-2;
 
+// the coarse solve, queued; its status stays in h->status
+int coarse_queue(rte_handle* h, const double* b, double* x, int nrhs) {
+    Scope sc(h, "coarse_cg");
+    // mixed modes at a loose tolerance (the default 0.3): the CG's E_c
+    // products in FP32, whose rounding lies orders below the tolerance
+    const bool f32 = h->mixed && h->opt.coarse_tol >= kCoarseF32Tol;
+    return coarse_cg(h->stream, h->d, b, x, nrhs, h->opt.coarse_tol, h->opt.coarse_maxit,
+                     h->cowork, h->cobytes, h->status, f32);
+}
+
 int coarse_inv(rte_handle* h, const double* b, double* x, int nrhs) {
-    {
-        Scope sc(h, "coarse_cg");
-        // mixed modes at a loose tolerance (the default 0.3): the CG's E_c
-        // products in FP32, whose rounding lies orders below the tolerance
-        const bool f32 = h->mixed && h->opt.coarse_tol >= kCoarseF32Tol;
-        RTE_TRY(coarse_cg(h->stream, h->d, b, x, nrhs, h->opt.coarse_tol, h->opt.coarse_maxit,
-                          h->cowork, h->cobytes, h->status, f32));
-    }
+    RTE_TRY(coarse_queue(h, b, x, nrhs));
     SolveStatus st;
     RTE_TRY(read_status(h, st));
     h->co_iters = st.iterations;
@@ -1437,14 +1452,47 @@ int apply_P1_pcg(rte_handle* h, const double* b, double* z, int nrhs) {
     return RTE_OK;
 }
 
+// The same in the mixed modes, whose inner applies take and give FP32: the
+// vector work in fused passes (kernels.cu).  Leaves z in FP32 in f1.
+int apply_P1_pcg_lo(rte_handle* h, const double* b, double* z, int nrhs) {
+    const DevSystem& d = h->d;
+    const size_t len = (size_t)d.nRp * d.nSp;
+    const int n = nrhs;
+    cudaStream_t s = h->stream;
+    double *R = h->e9, *P = h->e10, *Y = h->e6;
+    double *rho = h->sc + 8 * n, *alpha = h->sc + 10 * n, *beta = h->sc + 11 * n;
+    RTE_TRY(e0_inv(h, b, Y, n));                       // y = E_0^{-1} b
+    {
+        Scope sc(h, "axpy");
+        p1_start(s, b, Y, P, h->f1, len, n, h->partial, rho);
+    }
+    for (int k = 0; k < h->opt.l; ++k) {
+        const bool last = k + 1 == h->opt.l;
+        RTE_TRY(apply_E_lo(h, h->f1, h->f2, n, false));    // E p
+        {
+            Scope sc(h, "axpy");
+            p1_length(s, P, h->f2, len, n, h->partial, rho, alpha);
+            p1_step(s, alpha, k == 0, last, P, h->f2, k == 0 ? b : R, z, R, h->f1, len, n);
+        }
+        if (last) break;
+        RTE_TRY(e0_inv(h, R, Y, n));
+        Scope sc(h, "axpy");
+        p1_direction(s, R, Y, P, h->f1, len, n, h->partial, rho, beta);
+    }
+    return RTE_OK;
+}
+
 int apply_P1(rte_handle* h, const double* b, double* z, int nrhs) {
-    if (h->opt.p1_route == RTE_P1_PCG) return apply_P1_pcg(h, b, z, nrhs);
+    if (h->opt.p1_route == RTE_P1_PCG)
+        return h->mixed ? apply_P1_pcg_lo(h, b, z, nrhs) : apply_P1_pcg(h, b, z, nrhs);
     const DevSystem& d = h->d;
     const size_t len = (size_t)d.nRp * d.nSp;
     RTE_TRY(e0_inv(h, b, z, nrhs));   // z_1 = E_0^{-1} b
     for (int k = 1; k < h->opt.l; ++k) {
-        RTE_TRY(apply_E_inner(h, z, h->e5, nrhs, false));
-        {
+        if (!h->mixed) {
+            RTE_TRY(apply_E(h, z, h->e5, nrhs, false, b));
+        } else {
+            RTE_TRY(apply_E_inner(h, z, h->e5, nrhs, false));
             Scope sc(h, "axpy");
             axpby_per_rhs(h->stream, b, h->e5, len, nrhs, nullptr, -1.0, nullptr, 1.0);
         }
@@ -1459,11 +1507,11 @@ int apply_P1(rte_handle* h, const double* b, double* z, int nrhs) {
 // row (d^+ <= 16), in FP32 products on mixed handles (a preconditioner step:
 // its coarse solve stops at coarse_tol), in FP64 otherwise; the general
 // FP64 GEMM for larger d^+.
-int restrict_(rte_handle* h, const double* x, double* qc, int nrhs) {
+int restrict_(rte_handle* h, const double* x, double* qc, int nrhs, const float* sub = nullptr) {
     const DevSystem& d = h->d;
     Scope sc(h, "restrict");
     if (!restrict_rows(h->stream, nrhs * d.nRp, d.nSp, d.dP, x, d.WpN, h->mixed ? d.lo.WpN : nullptr,
-                       qc))
+                       qc, sub))
         gemm_f64(h->stream, nrhs * d.nRp, d.dP, d.nSp, x, d.nSp, d.WpN, d.dP, qc, d.dP, 1.0, 0.0,
                  0, nullptr, nullptr, nullptr, 1);
     return RTE_OK;
@@ -1479,19 +1527,41 @@ int prolong_add(rte_handle* h, const double* uc, double* x, int nrhs, double bet
     return RTE_OK;
 }
 
-// s = P_2 P_1 r = P_1 r + W E_c^{-1} W^T (r - (E - K^+) P_1 r)   (eq. product_pre)
-int precond(rte_handle* h, const double* r, double* s, int nrhs, bool p2) {
+// s = P_1 r and, with p2, the coarse residual's restriction solved into c2
+// (queued; its status is read by the caller): P_2 P_1 r = s + W c2
+int precond_queue(rte_handle* h, const double* r, double* s, int nrhs, bool p2) {
     const DevSystem& d = h->d;
     const size_t len = (size_t)d.nRp * d.nSp;
     RTE_TRY(apply_P1(h, r, s, nrhs));
-    if (!p2 || d.dP == 0) return RTE_OK;
-    RTE_TRY(apply_E_inner(h, s, h->e7, nrhs, true));
-    {
-        Scope sc(h, "axpy");   // e7 = r - (E - K^+) s
-        axpby_per_rhs(h->stream, r, h->e7, len, nrhs, nullptr, 1.0, nullptr, -1.0);
+    if (!p2) return RTE_OK;
+    if (h->mixed && h->opt.p1_route == RTE_P1_PCG && d.dP <= 16) {
+        // s in FP32 is in f1, and the restriction takes r - (E - K^+) s itself
+        RTE_TRY(apply_E_lo(h, h->f1, h->f2, nrhs, true));
+        RTE_TRY(restrict_(h, r, h->c1, nrhs, h->f2));
+    } else if (!h->mixed) {
+        // e7 = (E - K^+) s - r, and the sign goes into the coarse vector
+        RTE_TRY(apply_E(h, s, h->e7, nrhs, true, r));
+        RTE_TRY(restrict_(h, h->e7, h->c1, nrhs));
+        axpby_per_rhs(h->stream, nullptr, h->c1, (size_t)d.nRp * d.dP, nrhs, nullptr, 0.0, nullptr, -1.0);
+    } else {
+        RTE_TRY(apply_E_inner(h, s, h->e7, nrhs, true));
+        {
+            Scope sc(h, "axpy");   // e7 = r - (E - K^+) s
+            axpby_per_rhs(h->stream, r, h->e7, len, nrhs, nullptr, 1.0, nullptr, -1.0);
+        }
+        RTE_TRY(restrict_(h, h->e7, h->c1, nrhs));   // -q_c = W^T (r - (E-K) s)
     }
-    RTE_TRY(restrict_(h, h->e7, h->c1, nrhs));   // -q_c = W^T (r - (E-K) s)
-    RTE_TRY(coarse_inv(h, h->c1, h->c2, nrhs));  // -u_c
+    return coarse_queue(h, h->c1, h->c2, nrhs);  // -u_c
+}
+
+// s = P_2 P_1 r = P_1 r + W E_c^{-1} W^T (r - (E - K^+) P_1 r)   (eq. product_pre)
+int precond(rte_handle* h, const double* r, double* s, int nrhs, bool p2) {
+    p2 = p2 && h->d.dP > 0;
+    RTE_TRY(precond_queue(h, r, s, nrhs, p2));
+    if (!p2) return RTE_OK;
+    SolveStatus st;
+    RTE_TRY(read_status(h, st));
+    h->co_iters = st.iterations;
     // s <- s - W u_c, so that u_{n+1} = u_n - s = u_{n+1/2} + W u_c
     RTE_TRY(prolong_add(h, h->c2, s, nrhs, 1.0));
     return RTE_OK;
@@ -2307,29 +2377,38 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
     double* sv = h->e2;      // s = P_2 P_1 r
     double* rprev = h->e3;
     double* delta = h->e4;   // u_n - u_{n-1}
-    std::vector<double> hq(nrhs), hr(nrhs), hd1(nrhs), hd2(nrhs);
+    std::vector<double> hq(nrhs);
     double* sc = h->sc;
+    const bool p2 = d.dP > 0;
     dot_per_rhs(s, q, q, len, nrhs, h->partial, sc);
-    RTE_CUDA_TRY(cudaMemcpyAsync(hq.data(), sc, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
+    RTE_CUDA_TRY(cudaMemcpyAsync(h->host_sums, sc, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
     RTE_CUDA_TRY(cudaStreamSynchronize(s));
+    std::copy(h->host_sums, h->host_sums + nrhs, hq.begin());
     int it = 0, rc = RTE_OK;
     double worst = 0.0, energy = 0.0;
     for (it = 0;; ++it) {
         // r = (E - K^+) u - q   (Algorithm 3: residual)
         RTE_TRY(apply_E(h, u, r, nrhs, true, q));
-        dot_per_rhs(s, r, r, len, nrhs, h->partial, sc);
-        if (it > 0) {
-            // ||u_n - u_{n-1}||^2_{E-K} = delta^T (r_n - r_{n-1})
-            dot_per_rhs(s, delta, r, len, nrhs, h->partial, sc + nrhs);
-            dot_per_rhs(s, delta, rprev, len, nrhs, h->partial, sc + 2 * nrhs);
+        // ||r||^2 and ||u_n - u_{n-1}||^2_{E-K} = delta^T (r_n - r_{n-1})
+        {
+            Scope scp(h, "axpy");
+            residual_sums(s, r, it > 0 ? delta : nullptr, rprev, len, nrhs, h->partial, sc);
         }
-        RTE_CUDA_TRY(cudaMemcpyAsync(hr.data(), sc, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
-        if (it > 0) {
-            RTE_CUDA_TRY(cudaMemcpyAsync(hd1.data(), sc + nrhs, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
-            RTE_CUDA_TRY(cudaMemcpyAsync(hd2.data(), sc + 2 * nrhs, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
-        }
+        // the iteration's one synchronisation: its sums, and whether the
+        // solves queued since the last one gave up
+        RTE_CUDA_TRY(cudaMemcpyAsync(h->host_sums, sc, sizeof(double) * nrhs * (it > 0 ? 3 : 1),
+                                     cudaMemcpyDeviceToHost, s));
+        if (it > 0 && p2)
+            RTE_CUDA_TRY(cudaMemcpyAsync(h->host_status, h->status, sizeof(SolveStatus),
+                                         cudaMemcpyDeviceToHost, s));
+        if (it > 0 && d.e0_direct) RTE_TRY(e0_direct_error_fetch(s, h->host_e0_error));
         RTE_CUDA_TRY(cudaStreamSynchronize(s));
         settle_mk(h);
+        if (it > 0 && p2) {
+            if (h->host_status->timed_out) return fail(RTE_ERR_TIMEOUT, "a bounded grid barrier timed out");
+            h->co_iters = h->host_status->iterations;
+        }
+        const double *hr = h->host_sums, *hd1 = hr + nrhs, *hd2 = hd1 + nrhs;
         worst = 0.0;
         energy = 0.0;
         bool nan = false;
@@ -2340,20 +2419,29 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
             if (it > 0) energy = std::max(energy, std::sqrt(std::max(0.0, hd1[k] - hd2[k])));
         }
         if (stats && stats->history && it < stats->history_cap) stats->history[it] = worst;
-        if (d.e0_direct && it > 0) RTE_TRY(e0_direct_error(s));
+        if (it > 0 && d.e0_direct) RTE_TRY(e0_direct_error_check(s, *h->host_e0_error));
         if (nan) { rc = fail(RTE_ERR_DIVERGED, "residual is NaN or Inf"); break; }
         if (worst <= tol) break;
         if (it >= h->opt.max_iter) { rc = fail(RTE_ERR_MAXITER, "outer iteration cap reached"); break; }
-        // s = P_2 P_1 r ; u_{n+1} = u_n - s   (half step plus subspace correction)
-        RTE_TRY(precond(h, r, sv, nrhs, true));
-        RTE_CUDA_TRY(cudaMemcpyAsync(rprev, r, sizeof(double) * nrhs * len, cudaMemcpyDeviceToDevice, s));
-        RTE_CUDA_TRY(cudaMemcpyAsync(delta, sv, sizeof(double) * nrhs * len, cudaMemcpyDeviceToDevice, s));
-        {
-            Scope scp(h, "axpy");
-            k_neg<<<(unsigned)((nrhs * len + 255) / 256), 256, 0, s>>>(delta, nrhs * len);
-            count_launches(1);
-            axpby_per_rhs(s, sv, u, len, nrhs, nullptr, -1.0, nullptr, 1.0);
+        // s = P_2 P_1 r ; u_{n+1} = u_n - s   (half step plus subspace
+        // correction), delta = -s; the residuals' buffers change places
+        RTE_TRY(precond_queue(h, r, sv, nrhs, p2));
+        bool done = false;
+        if (p2) {
+            Scope scp(h, "prolong");
+            done = prolong_rows(s, nrhs * d.nRp, d.nSp, d.dP, h->c2, d.WpNT, h->mixed ? d.lo.WpNT : nullptr,
+                                sv, 1.0, u, delta, h->status);
         }
+        if (!done) {
+            if (p2) {
+                SolveStatus st;
+                RTE_TRY(read_status(h, st));
+                RTE_TRY(prolong_add(h, h->c2, sv, nrhs, 1.0));
+            }
+            Scope scp(h, "axpy");
+            update_solution(s, sv, u, delta, nrhs * len);
+        }
+        std::swap(r, rprev);
     }
     RTE_CUDA_TRY(cudaGetLastError());
     if (stats) {
@@ -2516,6 +2604,7 @@ void rte_destroy(rte_handle* h) {
     for (auto& kv : h->mk_graph) cudaGraphExecDestroy(kv.second);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->mk_state_host) cudaFreeHost(h->mk_state_host);
+    if (h->host_sums) cudaFreeHost(h->host_sums);
     for (void* p : h->allocs) cudaFreeAsync(p, h->stream);
     cudaStreamSynchronize(h->stream);
     // rte_destroy reports nothing: leave no error behind for the thread's
