@@ -4,8 +4,8 @@
 // built in h2_build.cpp.
 //
 // Every stage of the apply is one block-sparse product over 64-column
-// blocks, Out[:, blk j] (+)= sum_e In[:, blk in_e] B_e, with a 64 x 64 tile
-// of rows per block of threads (k_h2_bsr).  The blocks of threads are
+// blocks, Out[:, blk j] (+)= sum_e In[:, blk in_e] B_e, with a tile of up to
+// 64 rows and columns per block of threads (k_h2_bsr).  The blocks of threads are
 // ordered (group of 16 output blocks) x (row tile) x (output block), so that
 // the blocks running at one time share their B matrices and the input
 // columns of neighbouring clusters in L2.  Coupling matrices are not stored:
@@ -32,7 +32,6 @@ namespace rte {
 
 namespace {
 
-constexpr int kRT = 64;        // rows per tile of the block-sparse product
 constexpr int kGroup = 16;     // output blocks per raster group
 constexpr double kPi = 3.14159265358979323846;
 
@@ -226,26 +225,11 @@ __global__ void k_h2_to_f32(const double* __restrict__ x, float* __restrict__ y,
 }
 
 // ------------------------------------------------------------ apply
-template <typename T> struct Vec16;
-template <> struct Vec16<float> { using type = float4; static constexpr int n = 4; };
-template <> struct Vec16<double> { using type = double2; static constexpr int n = 2; };
-
-__device__ __forceinline__ void load4(const float* p, float* v) {
-    const float4 x = *reinterpret_cast<const float4*>(p);
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-}
-__device__ __forceinline__ void load4(const double* p, double* v) {
-    const double2 x = *reinterpret_cast<const double2*>(p);
-    const double2 y = *reinterpret_cast<const double2*>(p + 2);
-    v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
-}
-__device__ __forceinline__ void store4(float* p, const float* v) {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ void store4(double* p, const double* v) {
-    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
-    *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
-}
+// N consecutive values, read and written at once
+template <typename T, int N>
+struct alignas(sizeof(T) * N > 16 ? 16 : sizeof(T) * N) Vals {
+    T v[N];
+};
 
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
@@ -260,126 +244,153 @@ __device__ __forceinline__ double hg_t(double mu, double g, double c0) {
 }
 
 // Out[r, 64 out_blk[j] + q] (+)= sum_e sum_kk In[r, 64 in_blk[e] + kk] B_e[kk][q]
-// for a 64-row tile.  kMode 0: B_e = pool[mat[e]]; 1: its transpose;
-// 2: the coupling matrix 2 f k(s xi^out_q . xi^in_kk) with s = mat[e] the
-// part's sign and f = 1 (S^+) or s (S^-), zero outside the first k rows and
-// columns.  One block of 256 threads per (row tile, output block), each
-// thread a 4 x 4 piece of the 64 x 64 tile; the k sum in chunks of 256 bytes
-// per row staged in shared memory.
-template <typename T, int kMode, bool kAccum>
+// for a tile of TM rows and TN columns.  kMode 0: B_e = pool[mat[e]]; 1: its
+// transpose; 2: the coupling matrix 2 f k(s xi^out_q . xi^in_kk) with s =
+// mat[e] the part's sign and f = 1 (S^+) or s (S^-), zero outside the first k
+// rows and columns.  One block of 256 threads per (row tile, output block,
+// column tile), each thread a TM / 16 x TN / 16 piece of the tile; the k sum
+// in chunks of 256 bytes per row staged in shared memory, the next chunk's
+// loads in flight under the current one's products.  Every output sums over
+// (e, kk) in the same order whatever the tile.
+//
+// What bounds it: the FP32 (FP64) units once a call has thousands of tiles;
+// on a few hundred rows the longest chain of entries, on SMs most of which
+// have no tile at all (S^- of 1024 directions, 130 rows: 48 to 144 tiles of
+// 64 x 64 a stage).  bsr_tile takes the tile with the least work on the
+// busiest SM; A is read four values of k at a time, which takes the products
+// from shared memory's rate to the FP32 units'.  Measured, 130 rows of S^- on
+// 1024 directions, FP32: an apply 233 -> 176 us
+// (couplings 65 us, near field 115).
+template <typename T, int kMode, bool kAccum, int TM, int TN>
 __global__ void __launch_bounds__(256)
 k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict__ In,
          long long ldi, T* __restrict__ Out, long long ldo, const int* __restrict__ out_blk,
          const int* __restrict__ ptr, const int* __restrict__ in_blk, const int* __restrict__ mat,
          const T* __restrict__ pool, const T* __restrict__ xi, T g, T c0) {
-    using V = typename Vec16<T>::type;
-    constexpr int VN = Vec16<T>::n;
+    constexpr int VN = 16 / (int)sizeof(T);    // values per 16-byte vector
     constexpr int KC = 256 / (int)sizeof(T);   // 64 floats or 32 doubles per chunk
-    constexpr int VPR = KC / VN;               // 16-byte vectors per tile row
-    __shared__ __align__(16) T As[kRT][KC + VN];
-    __shared__ __align__(16) T Bs[KC][kH2B + VN];
-    __shared__ T xo[kH2B * 3], xin[kH2B * 3];
+    constexpr int VPR = KC / VN;               // vectors per tile row
+    constexpr int RM = TM / 16, CN = TN / 16;  // rows and columns per thread
+    constexpr int NCT = kH2B / TN, CPE = kH2B / KC;   // column tiles, chunks per entry
+    using V = Vals<T, VN>;
+    __shared__ __align__(16) T As[TM][KC + VN];
+    __shared__ __align__(16) T Bs[KC][TN + VN];
+    __shared__ T xo[TN * 3], xin[kH2B * 3];
 
     const long long bid = blockIdx.x;
-    const long long per = (long long)kGroup * rtiles;
+    const long long per = (long long)kGroup * NCT * rtiles;
     const int grp = (int)(bid / per);
     const long long rem = bid % per;
-    const int rt = (int)(rem / kGroup);
-    const int j = grp * kGroup + (int)(rem % kGroup);
+    const int rt = (int)(rem / (kGroup * NCT));
+    const int j = grp * kGroup + (int)(rem % (kGroup * NCT)) / NCT, q0 = (int)(rem % NCT) * TN;
     if (j >= nout) return;
-    const int r0 = rt * kRT;
+    const int r0 = rt * TM;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int ob = out_blk[j];
     if (kMode == 2)
-        for (int e = tid; e < kH2B * 3; e += 256) xo[e] = xi[(size_t)ob * kH2B * 3 + e];
+        for (int e = tid; e < TN * 3; e += 256) xo[e] = xi[((size_t)ob * kH2B + q0) * 3 + e];
 
-    T acc[4][4];
+    T acc[RM][CN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[i][q] = T(0);
+        for (int q = 0; q < CN; ++q) acc[i][q] = T(0);
 
-    for (int e = ptr[j]; e < ptr[j + 1]; ++e) {
-        const int ib = in_blk[e];
-        const int me = mat[e];
-        if (kMode == 2) {
-            __syncthreads();
-            for (int x = tid; x < kH2B * 3; x += 256) xin[x] = xi[(size_t)ib * kH2B * 3 + x];
-        }
-        for (int kc = 0; kc < kH2B; kc += KC) {
-            __syncthreads();
-            // A tile: 64 rows x KC columns of In
+    // chunk c: entry e0 + c / CPE, its inputs from kc = (c % CPE) KC
+    const int e0 = ptr[j], chunks = (ptr[j + 1] - e0) * CPE;
+    V av[RM], bv[kMode == 2 ? 1 : CN];
+    T xv = T(0);
+    int sign = 0;
+    auto load = [&](int c) {
+        const int e = e0 + c / CPE, kc = c % CPE * KC, ib = in_blk[e], me = mat[e];
 #pragma unroll
-            for (int s = 0; s < 4; ++s) {
-                const int idx = tid + 256 * s, row = idx / VPR, cv = idx % VPR;
-                V v;
-                if (r0 + row < rows)
-                    v = *reinterpret_cast<const V*>(In + (size_t)(r0 + row) * ldi +
+        for (int s = 0; s < RM; ++s) {   // TM rows x KC columns of In
+            const int idx = tid + 256 * s, row = idx / VPR, cv = idx % VPR;
+            if (r0 + row < rows)
+                av[s] = *reinterpret_cast<const V*>(In + (size_t)(r0 + row) * ldi +
                                                     (size_t)ib * kH2B + kc + cv * VN);
-                else
-                    memset(&v, 0, sizeof(V));
-                *reinterpret_cast<V*>(&As[row][cv * VN]) = v;
+            else
+                av[s] = V{};
+        }
+        if constexpr (kMode == 2) {
+            sign = me;
+            if (tid < kH2B * 3) xv = xi[(size_t)ib * kH2B * 3 + tid];
+        } else {   // KC rows (input index) x TN columns (output index), or transposed
+            const T* B = pool + (size_t)me * (kH2B * kH2B);
+#pragma unroll
+            for (int s = 0; s < CN; ++s) {
+                const int idx = tid + 256 * s;
+                bv[s] = kMode == 0
+                            ? *reinterpret_cast<const V*>(B + (size_t)(kc + idx / (TN / VN)) * kH2B +
+                                                          q0 + idx % (TN / VN) * VN)
+                            : *reinterpret_cast<const V*>(B + (size_t)(q0 + idx / VPR) * kH2B + kc +
+                                                          idx % VPR * VN);
             }
-            // B tile: KC rows (input index) x 64 columns (output index)
-            if (kMode == 0) {
-                const T* B = pool + (size_t)me * (kH2B * kH2B) + (size_t)kc * kH2B;
+        }
+    };
+    if (chunks > 0) load(0);
+    for (int c = 0; c < chunks; ++c) {
+        __syncthreads();   // the chunk before has been read
 #pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    const int idx = tid + 256 * s, br = idx / (kH2B / VN), bc = idx % (kH2B / VN);
-                    *reinterpret_cast<V*>(&Bs[br][bc * VN]) =
-                        *reinterpret_cast<const V*>(B + (size_t)br * kH2B + bc * VN);
+        for (int s = 0; s < RM; ++s) {
+            const int idx = tid + 256 * s;
+            *reinterpret_cast<V*>(&As[idx / VPR][idx % VPR * VN]) = av[s];
+        }
+        if constexpr (kMode == 2) {
+            const int me = sign, kc = c % CPE * KC;
+            if (tid < kH2B * 3) xin[tid] = xv;
+            __syncthreads();   // xin staged
+            const T f = T(2) * ((parity > 0 || me > 0) ? T(1) : T(-1));
+            const T sg = me > 0 ? T(1) : T(-1);
+            for (int idx = tid; idx < KC * TN; idx += 256) {
+                const int br = idx / TN, q = idx % TN, mu = kc + br;
+                T v = T(0);
+                if (mu < k && q0 + q < k) {
+                    const T d = xo[3 * q] * xin[3 * mu] + xo[3 * q + 1] * xin[3 * mu + 1] +
+                                xo[3 * q + 2] * xin[3 * mu + 2];
+                    v = f * hg_t(sg * d, g, c0);
                 }
-            } else if (kMode == 1) {
-                const T* B = pool + (size_t)me * (kH2B * kH2B);
+                Bs[br][q] = v;
+            }
+        } else {
 #pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    const int idx = tid + 256 * s, q = idx / VPR, cv = idx % VPR;
-                    const V v = *reinterpret_cast<const V*>(B + (size_t)q * kH2B + kc + cv * VN);
-                    const T* pv = reinterpret_cast<const T*>(&v);
+            for (int s = 0; s < CN; ++s) {
+                const int idx = tid + 256 * s;
+                if constexpr (kMode == 0) {
+                    *reinterpret_cast<V*>(&Bs[idx / (TN / VN)][idx % (TN / VN) * VN]) = bv[s];
+                } else {
 #pragma unroll
-                    for (int u = 0; u < VN; ++u) Bs[cv * VN + u][q] = pv[u];
-                }
-            } else {
-                __syncthreads();   // xin staged
-                const T f = T(2) * ((parity > 0 || me > 0) ? T(1) : T(-1));
-                const T sg = me > 0 ? T(1) : T(-1);
-                for (int idx = tid; idx < KC * kH2B; idx += 256) {
-                    const int br = idx / kH2B, q = idx % kH2B, mu = kc + br;
-                    T v = T(0);
-                    if (mu < k && q < k) {
-                        const T d = xo[3 * q] * xin[3 * mu] + xo[3 * q + 1] * xin[3 * mu + 1] +
-                                    xo[3 * q + 2] * xin[3 * mu + 2];
-                        v = f * hg_t(sg * d, g, c0);
-                    }
-                    Bs[br][q] = v;
+                    for (int u = 0; u < VN; ++u) Bs[idx % VPR * VN + u][idx / VPR] = bv[s].v[u];
                 }
             }
-            __syncthreads();
-#pragma unroll 8
-            for (int kk = 0; kk < KC; ++kk) {
-                T a[4], b[4];
+        }
+        __syncthreads();
+        if (c + 1 < chunks) load(c + 1);
+#pragma unroll 4
+        for (int k0 = 0; k0 < KC; k0 += VN) {
+            V a[RM];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[ty * 4 + i][kk];
-                load4(&Bs[kk][tx * 4], b);
+            for (int i = 0; i < RM; ++i) a[i] = *reinterpret_cast<const V*>(&As[ty * RM + i][k0]);
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+            for (int kk = 0; kk < VN; ++kk) {
+                const Vals<T, CN> w = *reinterpret_cast<const Vals<T, CN>*>(&Bs[k0 + kk][tx * CN]);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) acc[i][q] = fma_t(a[i], b[q], acc[i][q]);
+                for (int i = 0; i < RM; ++i)
+#pragma unroll
+                    for (int q = 0; q < CN; ++q) acc[i][q] = fma_t(a[i].v[kk], w.v[q], acc[i][q]);
             }
         }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = r0 + ty * 4 + i;
+    for (int i = 0; i < RM; ++i) {
+        const int r = r0 + ty * RM + i;
         if (r >= rows) continue;
-        T* o = Out + (size_t)r * ldo + (size_t)ob * kH2B + tx * 4;
-        if (kAccum) {
-            T old[4];
-            load4(o, old);
+        auto* o = reinterpret_cast<Vals<T, CN>*>(Out + (size_t)r * ldo + (size_t)ob * kH2B + q0 + tx * CN);
+        Vals<T, CN> w;
+        if (kAccum) w = *o;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[i][q] += old[q];
-        }
-        store4(o, acc[i]);
+        for (int q = 0; q < CN; ++q) w.v[q] = kAccum ? acc[i][q] + w.v[q] : acc[i][q];
+        *o = w;
     }
 }
 
@@ -634,19 +645,55 @@ int run_tc(cudaStream_t s, const DevList& L, int rows, const void* In, long long
     return RTE_OK;
 }
 
-template <typename T, int kMode, bool kAccum>
-int run_list(cudaStream_t s, const DevList& L, int rows, int k, int parity, const T* In,
+template <typename T, int kMode, bool kAccum, int TM, int TN>
+int run_tile(cudaStream_t s, const DevList& L, int rows, int k, int parity, const T* In,
              long long ldi, T* Out, long long ldo, const T* pool, const T* xi, double g) {
-    if (L.nout == 0 || rows == 0) return RTE_OK;
-    const int rtiles = (rows + kRT - 1) / kRT;
-    const long long grid = (long long)((L.nout + kGroup - 1) / kGroup) * kGroup * rtiles;
+    const int rtiles = (rows + TM - 1) / TM;
+    const long long grid = (long long)((L.nout + kGroup - 1) / kGroup) * kGroup * rtiles * (kH2B / TN);
     if (grid > 0x7fffffffLL) return fail(RTE_ERR_ARG, "H2 apply: too many rows for one launch");
     const T c0 = T((1.0 - g * g) / (4.0 * kPi));
-    k_h2_bsr<T, kMode, kAccum><<<(unsigned)grid, 256, 0, s>>>(
+    k_h2_bsr<T, kMode, kAccum, TM, TN><<<(unsigned)grid, 256, 0, s>>>(
         rows, rtiles, L.nout, k, parity, In, ldi, Out, ldo, L.out_blk, L.ptr, L.in_blk, L.mat, pool,
         xi, T(g), c0);
     count_launches(1);
     return RTE_OK;
+}
+
+// The tile of a call: TM = 64 or 32 rows, TN = 64 or 32 columns, whichever
+// gives the busiest SM the least work.  A tile's clocks per step of k, from
+// the FP32 units' rate (64 x 64: 32, 64 x 32: 16) or, below 64 rows, shared
+// memory's (20 and 12); in FP64 the units' two multiply-adds a clock; plus
+// the evaluation of a coupling matrix' TN entries per step.  Every column (or
+// row) tile more re-reads A (or B): a tenth on top, so that calls with many
+// tiles stay at 64 x 64.
+template <typename T>
+int bsr_tile(int nout, int rows, bool couple) {
+    const double sms = device_sm_count();
+    int best = 0;
+    double cost = 1e300;
+    for (int t = 0; t < 4; ++t) {
+        const int TM = t & 1 ? 32 : 64, TN = t & 2 ? 32 : 64;
+        double step = sizeof(T) == 8 ? TM * TN / 2 : TM == 64 ? TN / 2 : TN == 64 ? 20 : 12;
+        if (couple) step += (sizeof(T) == 8 ? 30 : 0.25) * TN;
+        const double blocks = (double)nout * ((rows + TM - 1) / TM) * (kH2B / TN);
+        const double c = std::ceil(blocks / sms) * step * (t ? 1.1 : 1.0);
+        if (c < cost) {
+            cost = c;
+            best = t;
+        }
+    }
+    return best;
+}
+
+template <typename T, int kMode, bool kAccum, typename... Args>
+int run_list(cudaStream_t s, const DevList& L, int rows, Args... args) {
+    if (L.nout == 0 || rows == 0) return RTE_OK;
+    switch (bsr_tile<T>(L.nout, rows, kMode == 2)) {
+        case 0: return run_tile<T, kMode, kAccum, 64, 64>(s, L, rows, args...);
+        case 1: return run_tile<T, kMode, kAccum, 32, 64>(s, L, rows, args...);
+        case 2: return run_tile<T, kMode, kAccum, 64, 32>(s, L, rows, args...);
+        default: return run_tile<T, kMode, kAccum, 32, 32>(s, L, rows, args...);
+    }
 }
 
 }  // namespace
