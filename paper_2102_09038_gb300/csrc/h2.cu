@@ -21,6 +21,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "device.h"
@@ -397,49 +398,69 @@ k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict_
 // ------------------------------------------------- tensor-core apply
 // The same block-sparse products on the tensor cores (tcgen05, BF16
 // operands, FP32 accumulation in tensor memory) for the BF16 apply.  One
-// block of 128 threads per (128-row tile, output block): warp 0 lane 0 loads
-// the A tile (128 rows x 64 columns of In, one 128-byte swizzled row per
-// matrix row) and the B tile (the 64 x 64 matrix, stored K-major as
-// Bt[output][input]) by TMA into a 4-stage ring, warp 1 lane 0 issues four
-// 128 x 64 x 16 MMAs per entry, and the four warps drain the 64 accumulator
-// columns.  Every wait is bounded (tc::mbar_wait).
+// block of 128 threads per (128-row tile, group of G output blocks): warp 0
+// lane 0 loads the A tile (128 rows x 64 columns of In, one 128-byte swizzled
+// row per matrix row) and the B tiles of the outputs that take this input
+// (64 x 64 matrices, stored K-major as Bt[output][input]) by TMA into a
+// 4-stage ring, warp 1 issues the MMAs, and the four warps drain 64 columns of
+// the accumulator per output.  Every wait is bounded (tc::mbar_wait).
+//
+// What bounds it: with G = 1 the reads from L2 (16 KB of A and 8 KB of B for
+// one 128 x 64 x 64 product; 80 % of L2's rate) and MMAs 64 columns wide (a
+// third of the tensor pipe).  The lists of neighbouring outputs (siblings in
+// the cluster tree) share nearly all their inputs: on the 16384-direction
+// sphere pairs of outputs have 14,500 distinct inputs between them in place of
+// 28,500, so G = 2 takes a third off the bytes and, where both take an input,
+// one MMA is 128 columns wide.  (G = 4, one block on an SM, left its ends
+// exposed: couplings 439 us.)  Every output's products keep the order of its
+// list.  Measured, S^+ of 16384 directions, 2048 rows: an apply 1366
+// -> 1074 us (couplings 429, near field 255); the near field, the last stage,
+// adds the far field's FP32 result and writes the FP64 one itself.
 constexpr int kTcRows = 128;
-constexpr int kTcStages = 4;
+constexpr int kTcGroup = 2;      // outputs per block where they share inputs
+__host__ __device__ constexpr int tc_stages(int G) { return G == 1 ? 4 : 3; }   // two blocks per SM
 constexpr uint32_t kTcABytes = kTcRows * tc::kRowBytes;   // 16 KB
-constexpr uint32_t kTcBBytes = kH2B * tc::kRowBytes;      // 8 KB
+constexpr uint32_t kTcBBytes = kH2B * tc::kRowBytes;      // 8 KB per output
 
-constexpr size_t tc_smem_bytes() {
-    return 1024 + (size_t)kTcStages * (kTcABytes + kTcBBytes) + (2 * kTcStages + 1) * 8 + 16;
+constexpr size_t tc_smem_bytes(int G) {
+    return 1024 + (size_t)tc_stages(G) * (kTcABytes + G * kTcBBytes);   // 1024: alignment
 }
 
-template <bool kAccum, typename TOut>
-__global__ void __launch_bounds__(128, 1)
+// out_blk [nout][G], mat [entry][G]: G = 1 the lists as they are; else -1
+// where a group is short or an output does not take the entry's input.  Old:
+// what the product is added to (null: nothing), Out itself or, for a result
+// in FP64, the FP32 array that holds it so far.
+template <int G, typename TOut>
+__global__ void __launch_bounds__(128, 2)
 k_h2_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-        int rows, int rtiles, int nout, TOut* __restrict__ Out, long long ldo,
-        const int* __restrict__ out_blk, const int* __restrict__ ptr,
+        int rows, int rtiles, int nout, const std::conditional_t<sizeof(TOut) == 8, float, TOut>* Old,
+        TOut* Out, long long ldo, const int* __restrict__ out_blk, const int* __restrict__ ptr,
         const int* __restrict__ in_blk, const int* __restrict__ mat) {
     using namespace tc;
-    constexpr uint32_t kTmemCols = kH2B;
+    constexpr int kTcStages = tc_stages(G);
+    constexpr uint32_t kTmemCols = G * kH2B;
+    constexpr int kRaster = kGroup / G;   // groups of a raster group
+    constexpr uint32_t kAll = (1u << G) - 1u;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sA = smem;
     uint8_t* sB = smem + kTcStages * kTcABytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + kTcStages * kTcBBytes);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kTcStages + 1);
+    __shared__ __align__(8) uint64_t bars[2 * kTcStages + 1];
+    __shared__ uint32_t tmem_slot, smask[kTcStages];   // smask: outputs of a stage's entry
 
     const long long bid = blockIdx.x;
-    const long long per = (long long)kGroup * rtiles;
+    const long long per = (long long)kRaster * rtiles;
     const int grp = (int)(bid / per);
     const long long rem = bid % per;
-    const int rt = (int)(rem / kGroup);
-    const int j = grp * kGroup + (int)(rem % kGroup);
+    const int rt = (int)(rem / kRaster);
+    const int j = grp * kRaster + (int)(rem % kRaster);
     if (j >= nout) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r0 = rt * kTcRows;
     const int e0 = ptr[j], steps = ptr[j + 1] - e0;
-    const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + kTcStages),
-                   done = smem_u32(bars + 2 * kTcStages);
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kTcStages,
+                   done = full0 + 16 * kTcStages;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kTcStages; ++s) {
             mbar_init(full0 + 8 * s, 1);
@@ -450,73 +471,129 @@ k_h2_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(tmem_slot)),
+                         smem_u32(&tmem_slot)),
                      "r"(kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = tmem_slot;
     bool ok = true;
 
     if (warp == 0 && lane == 0) {
-        for (int st = 0; st < steps && ok; ++st) {
-            const int s = st % kTcStages;
-            const uint32_t ph = (st / kTcStages) & 1;
-            if (!mbar_wait(empty0 + 8 * s, ph ^ 1)) { ok = false; break; }
-            mbar_expect_tx(full0 + 8 * s, kTcABytes + kTcBBytes);
-            tma_load_2d(smem_u32(sA + s * kTcABytes), &mapA, full0 + 8 * s, in_blk[e0 + st] * kH2B,
-                        r0);
-            tma_load_2d(smem_u32(sB + s * kTcBBytes), &mapB, full0 + 8 * s, 0, mat[e0 + st] * kH2B);
-        }
-    } else if (warp == 1 && lane == 0) {
-        const uint32_t idesc = (1u << 4)                               // D: FP32
-                               | (1u << 7) | (1u << 10)                // A, B: BF16
-                               | ((uint32_t)(kH2B >> 3) << 17)         // N = 64
-                               | ((uint32_t)(kTcRows >> 4) << 24);     // M = 128
-        for (int st = 0; st < steps && ok; ++st) {
-            const int s = st % kTcStages;
-            const uint32_t ph = (st / kTcStages) & 1;
-            if (!mbar_wait(full0 + 8 * s, ph)) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_u32(sA + s * kTcABytes), b0 = smem_u32(sB + s * kTcBBytes);
+        // the next entry's indices are read ahead of the wait for its stage
+        int in = 0, m[G];
+        auto entry = [&](int st) {
+            in = in_blk[e0 + st];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-                mma_issue(false, tmem, sw128_desc(a0 + 32 * kk), sw128_desc(b0 + 32 * kk), idesc,
-                          (st > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(empty0 + 8 * s);
+            for (int g = 0; g < G; ++g) m[g] = mat[(size_t)(e0 + st) * G + g];
+        };
+        if (steps > 0) entry(0);
+        int s = 0;
+        uint32_t ph = 1, loaded = 0;
+        for (int st = 0; st < steps; ++st) {
+            if (!mbar_wait(empty0 + 8 * s, ph)) { ok = false; break; }
+            uint32_t mask = 0;
+#pragma unroll
+            for (int g = 0; g < G; ++g) mask |= (m[g] >= 0 ? 1u : 0u) << g;
+            smask[s] = mask;
+            mbar_expect_tx(full0 + 8 * s, kTcABytes + __popc(mask) * kTcBBytes);
+            tma_load_2d(smem_u32(sA + s * kTcABytes), &mapA, full0 + 8 * s, in * kH2B, r0);
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (m[g] >= 0)
+                    tma_load_2d(smem_u32(sB + (s * G + g) * kTcBBytes), &mapB, full0 + 8 * s, 0,
+                                m[g] * kH2B);
+            loaded |= 1u << s;
+            if (++s == kTcStages) { s = 0; ph ^= 1; }
+            if (st + 1 < steps) entry(st + 1);
         }
-        mma_commit(done);
+        // after a timeout: the copies still in flight land before the block
+        // leaves (stages before s hold one of this round)
+        if (!ok)
+            for (int i = 0; i < kTcStages; ++i)
+                if (loaded >> i & 1u) mbar_wait(full0 + 8 * i, i < s ? ph ^ 1u : ph);
+    } else if (warp == 1) {
+        // the whole warp keeps warp-uniform values; one lane issues
+        constexpr uint32_t idesc = (1u << 4)                              // D: FP32
+                                   | (1u << 7) | (1u << 10)               // A, B: BF16
+                                   | ((uint32_t)(kH2B >> 3) << 17)        // N = 64
+                                   | ((uint32_t)(kTcRows >> 4) << 24);    // M = 128
+        constexpr uint32_t wide = idesc + ((uint32_t)((G - 1) * kH2B >> 3) << 17);   // N = 64 G
+        const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        uint32_t started = 0;   // outputs that hold a product already
+        int s = 0;
+        uint32_t ph = 0;
+        for (int st = 0; st < steps; ++st) {
+            if (!mbar_wait_warp(full0 + 8 * s, ph)) { ok = false; break; }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t mask = G == 1 ? 1u : __shfl_sync(0xffffffffu, smask[s], 0);
+            const uint64_t da = da0 + (uint64_t)(s * (kTcABytes >> 4)),
+                           db = db0 + (uint64_t)(s * (G * kTcBBytes >> 4));
+            if (mask == kAll && (started == 0u || started == kAll)) {
+                if (elect_one()) {
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        mma_issue(false, tm, da + 2 * kk, db + 2 * kk, wide,
+                                  (started || kk > 0) ? 1u : 0u);
+                }
+            } else {
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+                    if ((mask >> g & 1u) && elect_one()) {
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            mma_issue(false, tm + g * kH2B, da + 2 * kk,
+                                      db + (uint64_t)(g * (kTcBBytes >> 4)) + 2 * kk, idesc,
+                                      ((started >> g & 1u) || kk > 0) ? 1u : 0u);
+                    }
+            }
+            started |= mask;
+            __syncwarp();
+            if (elect_one()) mma_commit(empty0 + 8 * s);
+            if (++s == kTcStages) { s = 0; ph ^= 1; }
+        }
+        if (elect_one()) mma_commit(done);
     }
     __syncwarp();
     ok = mbar_wait(done, 0);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int row = r0 + warp * 32 + lane;
-    const int ob = out_blk[j];
-    for (int c0 = 0; c0 < kH2B; c0 += 16) {
+    for (int c0 = 0; c0 < G * kH2B; c0 += 16) {
+        const int ob = out_blk[(size_t)j * G + c0 / kH2B];
+        if (G > 1 && ob < 0) continue;
         float v[16];
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, v);
         if (!ok || row >= rows) continue;
         if (steps == 0)
             for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        TOut* dst = Out + (size_t)row * ldo + (size_t)ob * kH2B + c0;
-        if constexpr (sizeof(TOut) == 4) {
-            float4* d4 = reinterpret_cast<float4*>(dst);
+        const size_t at = (size_t)row * ldo + (size_t)ob * kH2B + c0 % kH2B;
+        if constexpr (sizeof(TOut) != 2) {
+            if (Old) {
+                const float4* o4 = reinterpret_cast<const float4*>(Old + at);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float4 w = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                if (kAccum) {
-                    const float4 o = d4[i];
-                    w.x += o.x; w.y += o.y; w.z += o.z; w.w += o.w;
+                for (int i = 0; i < 4; ++i) {
+                    const float4 o = o4[i];
+                    v[4 * i] += o.x; v[4 * i + 1] += o.y; v[4 * i + 2] += o.z; v[4 * i + 3] += o.w;
                 }
-                d4[i] = w;
+            }
+            if constexpr (sizeof(TOut) == 4) {
+                float4* d4 = reinterpret_cast<float4*>(Out + at);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    d4[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            } else {
+                double2* d2 = reinterpret_cast<double2*>(Out + at);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) d2[i] = make_double2(v[2 * i], v[2 * i + 1]);
             }
         } else {
-            uint4* d4 = reinterpret_cast<uint4*>(dst);
             uint32_t w[8];
-            if (kAccum) {
-                const uint4 o0 = d4[0], o1 = d4[1];
+            if (Old) {
+                const uint4* o4 = reinterpret_cast<const uint4*>(Old + at);
+                const uint4 o0 = o4[0], o1 = o4[1];
                 const uint32_t ow[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -530,6 +607,7 @@ k_h2_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtens
                 __nv_bfloat162 hv = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
                 w[i] = *reinterpret_cast<uint32_t*>(&hv);
             }
+            uint4* d4 = reinterpret_cast<uint4*>(Out + at);
             d4[0] = make_uint4(w[0], w[1], w[2], w[3]);
             d4[1] = make_uint4(w[4], w[5], w[6], w[7]);
         }
@@ -587,6 +665,11 @@ struct DevList {
     int *out_blk = nullptr, *ptr = nullptr, *in_blk = nullptr, *mat = nullptr;
 };
 
+// A list by groups of kTcGroup outputs (k_h2_tc), where that saves reads.
+struct TcList {
+    DevList one, group;
+};
+
 struct H2Parity {
     bool on = false;
     int m = 1;
@@ -599,50 +682,43 @@ struct H2Parity {
     // lists with matrix indices into that pool
     __nv_bfloat16* tcpool = nullptr;
     long long tc_total = 0;
-    DevList tc_up_leaf, tc_couple, tc_down_leaf, tc_near;
-    std::vector<DevList> tc_up, tc_down;
+    TcList tc_up_leaf, tc_couple, tc_down_leaf, tc_near;
+    std::vector<TcList> tc_up, tc_down;
 };
 
-int run_tc(cudaStream_t s, const DevList& L, int rows, const void* In, long long ldi,
-           const __nv_bfloat16* tcpool, long long tc_total, void* Out, long long ldo, bool out_f32,
-           bool accum) {
-    if (L.nout == 0 || rows == 0) return RTE_OK;
+template <int G, typename TOld, typename TOut>
+int launch_tc(cudaStream_t s, const CUtensorMap& ma, const CUtensorMap& mb, const DevList& L, int rows,
+              const TOld* Old, TOut* Out, long long ldo) {
+    auto kern = k_h2_tc<G, TOut>;
+    const size_t sm = tc_smem_bytes(G);
+    const int rtiles = (rows + kTcRows - 1) / kTcRows, raster = kGroup / G;
+    const long long grid = (long long)((L.nout + raster - 1) / raster) * raster * rtiles;
+    if (grid > 0x7fffffffLL) return fail(RTE_ERR_ARG, "H2 apply: too many rows for one launch");
+    // set on every call: the attribute is per device, and cheap to set
+    RTE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    kern<<<(unsigned)grid, 128, sm, s>>>(ma, mb, rows, rtiles, L.nout, Old, Out, ldo, L.out_blk, L.ptr,
+                                         L.in_blk, L.mat);
+    count_launches(1);
+    return RTE_OK;
+}
+
+// Out = Old + In B (Old null: In B)
+template <typename TOld, typename TOut>
+int run_tc(cudaStream_t s, const TcList& T, int rows, const void* In, long long ldi,
+           const __nv_bfloat16* tcpool, long long tc_total, const TOld* Old, TOut* Out, long long ldo) {
+    if (T.one.nout == 0 || rows == 0) return RTE_OK;
     CUtensorMap ma, mb;
     RTE_TRY(tc::make_map(&ma, In, false, rows, (int)ldi, kTcRows));
     RTE_TRY(tc::make_map(&mb, tcpool, false, (int)(tc_total * kH2B), kH2B, kH2B));
+    // groups when every SM gets two blocks twice over: below that single
+    // outputs keep more SMs busy than the shared reads save (an apply of S^+ of
+    // 16384 directions in groups against singly: 2048 rows 1067 us against
+    // 1203, 512 rows (664 groups) 374 against 389, 256 rows (332) 264 against
+    // 251; of 4096 directions, 1024 rows (304) 191 against 187)
     const int rtiles = (rows + kTcRows - 1) / kTcRows;
-    const long long grid = (long long)((L.nout + kGroup - 1) / kGroup) * kGroup * rtiles;
-    if (grid > 0x7fffffffLL) return fail(RTE_ERR_ARG, "H2 apply: too many rows for one launch");
-    const size_t sm = tc_smem_bytes();
-    static const bool attr = [sm] {
-        cudaFuncSetAttribute(k_h2_tc<false, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaFuncSetAttribute(k_h2_tc<true, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaFuncSetAttribute(k_h2_tc<false, __nv_bfloat16>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        cudaFuncSetAttribute(k_h2_tc<true, __nv_bfloat16>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        return true;
-    }();
-    (void)attr;
-    if (out_f32) {
-        float* o = static_cast<float*>(Out);
-        if (accum)
-            k_h2_tc<true, float><<<(unsigned)grid, 128, sm, s>>>(ma, mb, rows, rtiles, L.nout, o, ldo,
-                                                                 L.out_blk, L.ptr, L.in_blk, L.mat);
-        else
-            k_h2_tc<false, float><<<(unsigned)grid, 128, sm, s>>>(ma, mb, rows, rtiles, L.nout, o, ldo,
-                                                                  L.out_blk, L.ptr, L.in_blk, L.mat);
-    } else {
-        __nv_bfloat16* o = static_cast<__nv_bfloat16*>(Out);
-        if (accum)
-            k_h2_tc<true, __nv_bfloat16><<<(unsigned)grid, 128, sm, s>>>(
-                ma, mb, rows, rtiles, L.nout, o, ldo, L.out_blk, L.ptr, L.in_blk, L.mat);
-        else
-            k_h2_tc<false, __nv_bfloat16><<<(unsigned)grid, 128, sm, s>>>(
-                ma, mb, rows, rtiles, L.nout, o, ldo, L.out_blk, L.ptr, L.in_blk, L.mat);
-    }
-    count_launches(1);
-    return RTE_OK;
+    const bool group = T.group.nout > 0 && (long long)T.group.nout * rtiles >= 4 * device_sm_count();
+    return group ? launch_tc<kTcGroup>(s, ma, mb, T.group, rows, Old, Out, ldo)
+                 : launch_tc<1>(s, ma, mb, T.one, rows, Old, Out, ldo);
 }
 
 template <typename T, int kMode, bool kAccum, int TM, int TN>
@@ -848,11 +924,20 @@ int build_tc(rte_h2* h, int q, const rte::H2Lists& lists, cudaStream_t s) {
                                                    hp.couple.in_blk, hp.couple.mat, hp.tcpool, C0);
     count_launches((src.empty() ? 0 : 1) + (F > 0 ? 1 : 0));
     // the lists with tensor-core matrix indices
-    auto remap = [&](const H2List& l, long long base, long long from, DevList& d) {
+    auto remap = [&](const H2List& l, long long base, long long from, TcList& d) -> int {
         H2List c = l;
         for (size_t e = 0; e < c.mat.size(); ++e)
             c.mat[e] = (int)(base + (from < 0 ? (long long)e : c.mat[e] - from));
-        return upload_list(h, c, d, s);
+        RTE_TRY(upload_list(h, c, d.one, s));
+        const H2List g = h2_group_list(c, kTcGroup);
+        // tiles read by groups (a 16 KB input, 8 KB matrices) against singly
+        // where blocks have entries enough to hide their ends
+        if (2 * g.in_blk.size() + c.in_blk.size() < 0.8 * 3 * c.in_blk.size() &&
+            g.in_blk.size() >= 8 * g.ptr.size()) {
+            RTE_TRY(upload_list(h, g, d.group, s));
+            d.group.nout /= kTcGroup;
+        }
+        return RTE_OK;
     };
     RTE_TRY(remap(lists.up_leaf, Vt0, pl.leaf0, hp.tc_up_leaf));
     RTE_TRY(remap(lists.down_leaf, V0, pl.leaf0, hp.tc_down_leaf));
@@ -1130,19 +1215,19 @@ int rte_h2_apply(rte_h2* h, int parity, int precision, const double* X, double* 
             wb + ((2 * (size_t)rows * nh + (size_t)rows * ncols) * 2 + 255) / 256 * 256);
         const long long ldx = (long long)ncols, ldh = (long long)nh;
         convert(s, X, Xb, (size_t)rows * ncols);
-        RTE_TRY(run_tc(s, hp.tc_up_leaf, rows, Xb, ldx, hp.tcpool, hp.tc_total, Xh, ldh, false, false));
+        const __nv_bfloat16* none = nullptr;
+        RTE_TRY(run_tc(s, hp.tc_up_leaf, rows, Xb, ldx, hp.tcpool, hp.tc_total, none, Xh, ldh));
         for (int d = P.ld - 1; d >= P.dmin; --d)
-            RTE_TRY(run_tc(s, hp.tc_up[d - P.dmin], rows, Xh, ldh, hp.tcpool, hp.tc_total, Xh, ldh,
-                           false, false));
+            RTE_TRY(run_tc(s, hp.tc_up[d - P.dmin], rows, Xh, ldh, hp.tcpool, hp.tc_total, none, Xh, ldh));
         cudaMemsetAsync(Yh, 0, (size_t)rows * nh * 2, s);
-        RTE_TRY(run_tc(s, hp.tc_couple, rows, Xh, ldh, hp.tcpool, hp.tc_total, Yh, ldh, false, false));
+        RTE_TRY(run_tc(s, hp.tc_couple, rows, Xh, ldh, hp.tcpool, hp.tc_total, none, Yh, ldh));
         for (int d = P.dmin; d < P.ld; ++d)
-            RTE_TRY(run_tc(s, hp.tc_down[d - P.dmin], rows, Yh, ldh, hp.tcpool, hp.tc_total, Yh, ldh,
-                           false, true));
-        RTE_TRY(run_tc(s, hp.tc_down_leaf, rows, Yh, ldh, hp.tcpool, hp.tc_total, Y32, ldx, true,
-                       false));
-        RTE_TRY(run_tc(s, hp.tc_near, rows, Xb, ldx, hp.tcpool, hp.tc_total, Y32, ldx, true, true));
-        convert(s, Y32, Y, (size_t)rows * ncols);
+            RTE_TRY(run_tc(s, hp.tc_down[d - P.dmin], rows, Yh, ldh, hp.tcpool, hp.tc_total, Yh, Yh, ldh));
+        RTE_TRY(run_tc(s, hp.tc_down_leaf, rows, Yh, ldh, hp.tcpool, hp.tc_total,
+                       (const float*)nullptr, Y32, ldx));
+        // every output block has a near list (a leaf is near itself): the last
+        // stage writes the result
+        RTE_TRY(run_tc(s, hp.tc_near, rows, Xb, ldx, hp.tcpool, hp.tc_total, Y32, Y, ldx));
         // the pipelines' bounded waits: read the timeout flag (synchronises)
         int flag = 0;
         RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(&flag, tc::g_tc_error, sizeof(int), 0,

@@ -68,6 +68,12 @@ struct H2Lists {
 };
 void h2_lists(const H2Plan& P, const H2Pool& pool, H2Lists& L);
 
+// The list by groups of G consecutive outputs: ptr per group, out_blk [group][G]
+// and mat [entry][G], -1 where a group is short or an output does not take the
+// entry's input.  Every output meets its entries in the list's order.  Empty
+// when an output has no entries.
+H2List h2_group_list(const H2List& l, int G);
+
 // Limit of one mbarrier wait of the tensor-core H^2 products (SM cycles).
 int h2_set_wait_cycles(long long cycles);
 

@@ -209,4 +209,54 @@ void h2_lists(const H2Plan& P, const H2Pool& pool, H2Lists& L) {
         }
 }
 
+H2List h2_group_list(const H2List& l, int G) {
+    H2List g;
+    g.ptr.push_back(0);
+    const int nout = (int)l.out_blk.size();
+    for (int j0 = 0; j0 < nout; j0 += G) {
+        const int n = std::min(G, nout - j0);
+        std::vector<int> at(n);
+        std::vector<std::map<int, int>> left(n);   // inputs a list still has to take
+        for (int q = 0; q < n; ++q) {
+            at[q] = l.ptr[j0 + q];
+            if (at[q] == l.ptr[j0 + q + 1]) return H2List();
+            for (int e = at[q]; e < l.ptr[j0 + q + 1]; ++e) ++left[q][l.in_blk[e]];
+        }
+        auto live = [&](int q) { return at[q] < l.ptr[j0 + q + 1]; };
+        auto head = [&](int q) { return l.in_blk[at[q]]; };
+        for (;;) {
+            // the next input: one that every list still to take it has next,
+            // and if there is none the one most lists have next
+            int best = -1, score = -1;
+            for (int q = 0; q < n; ++q) {
+                if (!live(q)) continue;
+                int takes = 0, waits = 0;
+                for (int r = 0; r < n; ++r) {
+                    if (!live(r)) continue;
+                    if (head(r) == head(q)) ++takes;
+                    else if (left[r].count(head(q)) && left[r][head(q)] > 0) ++waits;
+                }
+                const int sc = (waits == 0 ? G : 0) + takes;
+                if (sc > score) {
+                    score = sc;
+                    best = head(q);
+                }
+            }
+            if (best < 0) break;
+            g.in_blk.push_back(best);
+            for (int q = 0; q < G; ++q) {
+                const bool take = q < n && live(q) && head(q) == best;
+                g.mat.push_back(take ? l.mat[at[q]] : -1);
+                if (take) {
+                    --left[q][best];
+                    ++at[q];
+                }
+            }
+        }
+        for (int q = 0; q < G; ++q) g.out_blk.push_back(q < n ? l.out_blk[j0 + q] : -1);
+        g.ptr.push_back((int)g.in_blk.size());
+    }
+    return g;
+}
+
 }  // namespace rte
