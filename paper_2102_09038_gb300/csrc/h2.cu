@@ -260,8 +260,9 @@ __device__ __forceinline__ double hg_t(double mu, double g, double c0) {
 // 64 x 64 a stage).  bsr_tile takes the tile with the least work on the
 // busiest SM; A is read four values of k at a time, which takes the products
 // from shared memory's rate to the FP32 units'.  Measured, 130 rows of S^- on
-// 1024 directions, FP32: an apply 233 -> 176 us
-// (couplings 65 us, near field 115).
+// 1024 directions, FP32: an apply 231 -> 169 us
+// (couplings 29 us, 65 before an entry's indices were read a chunk ahead of
+// its loads; near field 106).
 template <typename T, int kMode, bool kAccum, int TM, int TN>
 __global__ void __launch_bounds__(256)
 k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict__ In,
@@ -302,8 +303,14 @@ k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict_
     V av[RM], bv[kMode == 2 ? 1 : CN];
     T xv = T(0);
     int sign = 0;
+    // the entry's indices are read one chunk ahead of the loads that use them
+    int ib_next = chunks > 0 ? in_blk[e0] : 0, me_next = chunks > 0 ? mat[e0] : 0;
     auto load = [&](int c) {
-        const int e = e0 + c / CPE, kc = c % CPE * KC, ib = in_blk[e], me = mat[e];
+        const int kc = c % CPE * KC, ib = ib_next, me = me_next;
+        if (c + 1 < chunks) {
+            ib_next = in_blk[e0 + (c + 1) / CPE];
+            me_next = mat[e0 + (c + 1) / CPE];
+        }
 #pragma unroll
         for (int s = 0; s < RM; ++s) {   // TM rows x KC columns of In
             const int idx = tid + 256 * s, row = idx / VPR, cv = idx % VPR;
