@@ -292,7 +292,9 @@ def roofline_of(name, total_ms, launches, d, nrhs, info, peaks, src, fp64_peak, 
     """Roofline of one timing scope: the algorithmic work of one launch
     (kernel_work) over the scope's mean launch time, against the measured
     peak of its bound; fp64_peak() gives the measured FP64 rate (timed only
-    when a scope needs it)."""
+    when a scope needs it).  The algorithmic counts are of the method's dense
+    steps; where the library does
+    less, performed_work says how much (performed, performed_frac)."""
     avg_ms = total_ms / max(launches, 1)
     roof = dict(kernel=name, bound=None, achieved=None, peak=None, unit=None, frac=None,
                 launches=launches, avg_ms=avg_ms)
@@ -319,7 +321,39 @@ def roofline_of(name, total_ms, launches, d, nrhs, info, peaks, src, fp64_peak, 
         if impl is not None:
             roof.update(impl_bytes=impl,
                         impl_frac=impl / (avg_ms / 1e3) / 1e9 / peaks['hbm_gbs'])
+    done = performed_work(name, d, nrhs, tol)
+    if done is not None:
+        roof.update(performed=done, performed_frac=roof['frac'] * done / amount)
     return roof
+
+
+def performed_work(name, d, nrhs, tol):
+    """The work one launch of a scope performs where that is less than
+    kernel_work's dense count, in the same unit (else None):
+      * FP64 contractions of (M^- - K^-)^{-1}: between the two spatial
+        derivatives and the eigenbasis, 2 n_S^+ for 3 n_S^+ on one side;
+      * the FP64 transport and its transpose: two derivatives per cell and
+        direction in place of three odd values;
+      * E_0 direct: the upper-triangle tiles (8 x 8) of each row's inverse and
+        its coupling coefficients, read twice per sweep of four right-hand
+        sides, plus the right-hand side and the solution."""
+    nRp, nRm, nS, nSm = d['nRp'], d['nRm'], d['nSp'], d['nSm']
+    if name in ('gemm_mk_eig1', 'gemm_mk_eig2'):
+        return 2.0 * nrhs * nRm * nSm * 2 * nS
+    if name in ('dgemm_split_mk1', 'dgemm_split_mk2') and tol:
+        S = split_slices_for(tol)
+        return S * (S + 1) // 2 * 2.0 * nrhs * nRm * nSm * 2 * nS
+    if name == 'transport_A':
+        return 8.0 * nrhs * (nRp * nS + nRm * 2 * nS)
+    if name == 'apply_even':
+        return 8.0 * nrhs * (nRm * 2 * nS + 4 * nRp * nS)
+    if name in ('e0_direct', 'e0_direct64'):
+        w = 8 if name == 'e0_direct64' else 4
+        nt = (d['mesh'] + 8) // 8
+        rec = 64 * (nt * (nt + 1) // 2) + 2 * ((16 * nt + 63) // 64 * 64)
+        return (2.0 * nS * (d['mesh'] + 1) * rec * w * ((nrhs + 3) // 4)
+                + 32.0 * nRp * nrhs * nS)
+    return None
 
 
 def scope_rooflines(tim, d, nrhs, info, peaks, src, fp64_peak, tol, count=4):
@@ -335,8 +369,9 @@ def scope_rooflines(tim, d, nrhs, info, peaks, src, fp64_peak, tol, count=4):
 
 
 def kernel_impl_bytes(name, d, nrhs, info):
-    """The bytes the E_0 kernels move by their own design, per launch (kept
-    beside the algorithmic count): per V-cycle and active (node, column) the
+    """The bytes of the E_0 kernels' own design, per launch (kept beside the
+    algorithmic count; the direct route's are those of dense padded rows,
+    performed_work has what its packed records move): per V-cycle and active (node, column) the
     12 CG-vector passes of the precision w and the iterate read and written,
     the V-cycle's 17 FP32 array passes per level (4^-l of the level-0 size)
     and the coarsest level's dense per-direction inverses, plus the FP64
