@@ -907,7 +907,8 @@ k_p1_step(const double* __restrict__ alpha, int first, int last, const double* _
     const double a = alpha[blockIdx.y];
     for (size_t e = ((size_t)blockIdx.x * 256 + threadIdx.x) * W; e < len; e += (size_t)gridDim.x * 256 * W) {
         const Pack<double, W> p = *reinterpret_cast<const Pack<double, W>*>(P + o + e);
-        Pack<double, W> z;
+        Pack<double, W> z, b;
+        if (!last) b = *reinterpret_cast<const Pack<double, W>*>(B + o + e);   // before Z, which may be B
         if (!first) z = *reinterpret_cast<const Pack<double, W>*>(Z + o + e);
 #pragma unroll
         for (int w = 0; w < W; ++w) z.v[w] = first ? a * p.v[w] : a * p.v[w] + z.v[w];
@@ -918,7 +919,6 @@ k_p1_step(const double* __restrict__ alpha, int first, int last, const double* _
             for (int w = 0; w < W; ++w) f.v[w] = (float)z.v[w];
             *reinterpret_cast<Pack<float, W>*>(F + o + e) = f;
         } else {
-            Pack<double, W> b = *reinterpret_cast<const Pack<double, W>*>(B + o + e);
             const Pack<float, W> g = *reinterpret_cast<const Pack<float, W>*>(F2 + o + e);
 #pragma unroll
             for (int w = 0; w < W; ++w) b.v[w] = -a * (double)g.v[w] + b.v[w];

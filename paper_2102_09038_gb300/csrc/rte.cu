@@ -1461,6 +1461,12 @@ int apply_P1_pcg_lo(rte_handle* h, const double* b, double* z, int nrhs) {
     cudaStream_t s = h->stream;
     double *R = h->e9, *P = h->e10, *Y = h->e6;
     double *rho = h->sc + 8 * n, *alpha = h->sc + 10 * n, *beta = h->sc + 11 * n;
+    // the multigrid route reads its right-hand side 16 bytes at a time: a
+    // caller's vector that is not aligned for that is copied first
+    if (!d.e0_direct && (reinterpret_cast<uintptr_t>(b) & 15)) {
+        RTE_CUDA_TRY(cudaMemcpyAsync(R, b, sizeof(double) * n * len, cudaMemcpyDeviceToDevice, s));
+        b = R;
+    }
     RTE_TRY(e0_inv(h, b, Y, n));                       // y = E_0^{-1} b
     {
         Scope sc(h, "axpy");

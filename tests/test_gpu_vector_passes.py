@@ -52,3 +52,40 @@ def test_unaligned_vectors(m, levels, nrhs, n_plus, precision):
             assert res.max().item() <= 2e-9
     finally:
         s.close()
+
+
+@pytest.mark.parametrize('precision', [1, 2])
+def test_unaligned_vectors_on_the_multigrid_route(precision):
+    # that route reads its right-hand side 16 bytes at a time; E_0 CG to 1e-5,
+    # so the two results agree to a few times that
+    import paper_2102_09038_gb300 as rte
+    m, levels, nrhs = 9, 2, 2
+    p = workloads.constant(m, levels, 0.6, 1.5, 1.2)
+    s = rte.Solver(p, n_plus=2, n_minus=3, precision=precision, max_rhs=nrhs,
+                   e0_route=rte.E0_MULTIGRID, e0_tol=1e-5)
+    try:
+        x = np.random.default_rng(m).standard_normal((nrhs, (m + 1) ** 2, 4 << (2 * levels)))
+        got = []
+        for by_in, by_out in ((0, 0), (1, 0), (0, 1), (1, 1)):
+            out = shifted(np.zeros_like(x), by_out)
+            s.precond(shifted(x, by_in), False, out)
+            got.append(out.cpu().numpy())
+        for g in got[1:]:
+            assert np.abs(g - got[0]).max() <= 1e-4 * np.abs(got[0]).max()
+    finally:
+        s.close()
+
+
+def test_p1_in_place():
+    # the P_1 steps alone may write their result over their argument
+    import paper_2102_09038_gb300 as rte
+    p = workloads.constant(9, 2, 0.6, 1.5, 1.2)
+    s = rte.Solver(p, n_plus=2, n_minus=3, precision=rte.MIXED_BF16, max_rhs=2)
+    try:
+        x = np.random.default_rng(5).standard_normal((2, 100, 64))
+        want = s.precond(shifted(x, 0), False)
+        got = shifted(x, 0)
+        s.precond(got, False, got)
+        assert (got - want).abs().max().item() <= 1e-7 * want.abs().max().item()
+    finally:
+        s.close()
