@@ -127,10 +127,10 @@ struct SolveStatus {
 //   0: none
 //   1: 1 / (at[r % rows] - lam[c] * as[r % rows])           eigenbasis of M-K
 //   2: 1 / (at - lam as) - 1 / at                            Lemma precond.
-void gemm_f64(cudaStream_t s, int M, int N, int K, const double* A, int lda,
-              const double* B, int ldb, double* C, int ldc, double alpha,
-              double beta, int epi, const double* at, const double* as,
-              const double* lam, int rows);
+int gemm_f64(cudaStream_t s, int M, int N, int K, const double* A, int lda,
+             const double* B, int ldb, double* C, int ldc, double alpha,
+             double beta, int epi, const double* at, const double* as,
+             const double* lam, int rows);
 
 // Z = A U (eq. AR): even (nrhs x nRp x nSp) -> odd (nrhs x nRm x nSm)
 void apply_A(cudaStream_t s, const DevSystem& d, const double* U, double* Z,

@@ -49,7 +49,10 @@ k_gemm_f64(int M, int N, int K, const double* __restrict__ A, int lda,
     __shared__ double As[16][TM + 1];
     __shared__ double Bs[16][TN + 2];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+    // one-dimensional grid, column tiles fastest: the row tiles of a tall call
+    // (one per 16 rows of nrhs n_R^-) exceed the 65535 of the grid's y
+    const int ntn = (N + TN - 1) / TN;
+    const int m0 = (int)(blockIdx.x / ntn) * TM, n0 = (int)(blockIdx.x % ntn) * TN;
     double acc[RM][RN], a[RM], b[RN];
 #pragma unroll
     for (int i = 0; i < RM; ++i)
@@ -1070,7 +1073,7 @@ int device_sm_count() {
 }
 
 template <int EPI, typename... Args>
-static void gemm_f64_epi(cudaStream_t s, int M, int N, Args... args) {
+static int gemm_f64_epi(cudaStream_t s, int M, int N, Args... args) {
     // products on the busiest SM, per step of K; a little more for the
     // operand traffic of each smaller tile
     const int tiles[4][2] = {{64, 64}, {32, 64}, {32, 32}, {16, 32}};
@@ -1085,24 +1088,29 @@ static void gemm_f64_epi(cudaStream_t s, int M, int N, Args... args) {
             best = t;
         }
     }
-    const dim3 grid((N + tiles[best][1] - 1) / tiles[best][1], (M + tiles[best][0] - 1) / tiles[best][0]);
+    const long long grid = ((N + tiles[best][1] - 1LL) / tiles[best][1]) *
+                           ((M + tiles[best][0] - 1LL) / tiles[best][0]);
+    if (grid > 0x7fffffffLL) return fail(RTE_ERR_ARG, "FP64 GEMM: too many tiles for one launch");
+    const unsigned g = (unsigned)grid;
     switch (best) {
-        case 0: k_gemm_f64<EPI, 64, 64><<<grid, 256, 0, s>>>(M, N, args...); break;
-        case 1: k_gemm_f64<EPI, 32, 64><<<grid, 256, 0, s>>>(M, N, args...); break;
-        case 2: k_gemm_f64<EPI, 32, 32><<<grid, 256, 0, s>>>(M, N, args...); break;
-        default: k_gemm_f64<EPI, 16, 32><<<grid, 256, 0, s>>>(M, N, args...); break;
+        case 0: k_gemm_f64<EPI, 64, 64><<<g, 256, 0, s>>>(M, N, args...); break;
+        case 1: k_gemm_f64<EPI, 32, 64><<<g, 256, 0, s>>>(M, N, args...); break;
+        case 2: k_gemm_f64<EPI, 32, 32><<<g, 256, 0, s>>>(M, N, args...); break;
+        default: k_gemm_f64<EPI, 16, 32><<<g, 256, 0, s>>>(M, N, args...); break;
     }
+    RTE_CUDA_TRY(cudaGetLastError());
+    return RTE_OK;
 }
 
-void gemm_f64(cudaStream_t s, int M, int N, int K, const double* A, int lda,
-              const double* B, int ldb, double* C, int ldc, double alpha,
-              double beta, int epi, const double* at, const double* as,
-              const double* lam, int rows) {
-    if (M <= 0 || N <= 0) return;
+int gemm_f64(cudaStream_t s, int M, int N, int K, const double* A, int lda,
+             const double* B, int ldb, double* C, int ldc, double alpha,
+             double beta, int epi, const double* at, const double* as,
+             const double* lam, int rows) {
+    if (M <= 0 || N <= 0) return RTE_OK;
     count_launches(1);
-    if (epi == 1) gemm_f64_epi<1>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
-    else if (epi == 2) gemm_f64_epi<2>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
-    else gemm_f64_epi<0>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
+    if (epi == 1) return gemm_f64_epi<1>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
+    if (epi == 2) return gemm_f64_epi<2>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
+    return gemm_f64_epi<0>(s, M, N, K, A, lda, B, ldb, C, ldc, alpha, beta, at, as, lam, rows);
 }
 
 void apply_A(cudaStream_t s, const DevSystem& d, const double* U, double* Z, int nrhs) {

@@ -980,13 +980,13 @@ int mk_inv_eigen(rte_handle* h, const double* Z1, double* Z2, int nrhs) {
     }
     {
         Scope sc(h, "gemm_mk_eig1");
-        gemm_f64(h->stream, rows, d.nSm, d.nSm, Z1, d.nSm, d.Vm, d.nSm, h->z4, d.nSm, 1.0,
-                 0.0, 1, d.cell_at, d.cell_as, d.lamM, d.nRm);
+        RTE_TRY(gemm_f64(h->stream, rows, d.nSm, d.nSm, Z1, d.nSm, d.Vm, d.nSm, h->z4, d.nSm, 1.0,
+                         0.0, 1, d.cell_at, d.cell_as, d.lamM, d.nRm));
     }
     {
         Scope sc(h, "gemm_mk_eig2");
-        gemm_f64(h->stream, rows, d.nSm, d.nSm, h->z4, d.nSm, d.VmT, d.nSm, Z2, d.nSm, 1.0,
-                 0.0, 0, nullptr, nullptr, nullptr, 1);
+        RTE_TRY(gemm_f64(h->stream, rows, d.nSm, d.nSm, h->z4, d.nSm, d.VmT, d.nSm, Z2, d.nSm, 1.0,
+                         0.0, 0, nullptr, nullptr, nullptr, 1));
     }
     return RTE_OK;
 }
@@ -1012,8 +1012,8 @@ int mk_first(rte_handle* h, const double* G, int nrhs) {
         return RTE_OK;
     }
     Scope sc(h, "gemm_mk_eig1");
-    gemm_f64(h->stream, rows, d.nSm, n2, G, n2, d.Wg, d.nSm, h->z4, d.nSm, 1.0, 0.0, 1, d.cell_at,
-             d.cell_as, d.lamM, d.nRm);
+    RTE_TRY(gemm_f64(h->stream, rows, d.nSm, n2, G, n2, d.Wg, d.nSm, h->z4, d.nSm, 1.0, 0.0, 1, d.cell_at,
+                     d.cell_as, d.lamM, d.nRm));
     return RTE_OK;
 }
 
@@ -1033,8 +1033,8 @@ int mk_second(rte_handle* h, double* out, int nrhs, bool odd) {
                           odd ? d.ex_Vm : d.ex_Wg, N, d.nSm, S, out, N, 0, nullptr, 1, d.split_S);
     }
     Scope sc(h, "gemm_mk_eig2");
-    gemm_f64(h->stream, rows, N, d.nSm, h->z4, d.nSm, odd ? d.VmT : d.WgT, N, out, N, 1.0, 0.0, 0,
-             nullptr, nullptr, nullptr, 1);
+    RTE_TRY(gemm_f64(h->stream, rows, N, d.nSm, h->z4, d.nSm, odd ? d.VmT : d.WgT, N, out, N, 1.0, 0.0, 0,
+                     nullptr, nullptr, nullptr, 1));
     return RTE_OK;
 }
 
@@ -1044,11 +1044,11 @@ int mk_prec(rte_handle* h, const double* B, double* X, double* tmp, int nrhs) {
     const DevSystem& d = h->d;
     const int rows = nrhs * d.nRm;
     Scope sc(h, "mk_prec");
-    gemm_f64(h->stream, rows, d.dM, d.nSm, B, d.nSm, d.WmN, d.dM, tmp, d.dM, 1.0, 0.0, 2,
-             d.cell_at, d.cell_as, d.lamM, d.nRm);
+    RTE_TRY(gemm_f64(h->stream, rows, d.dM, d.nSm, B, d.nSm, d.WmN, d.dM, tmp, d.dM, 1.0, 0.0, 2,
+                     d.cell_at, d.cell_as, d.lamM, d.nRm));
     mk_minv_scale(h->stream, d, B, X, nrhs);
-    gemm_f64(h->stream, rows, d.nSm, d.dM, tmp, d.dM, d.WmNT, d.nSm, X, d.nSm, 1.0, 1.0, 0,
-             nullptr, nullptr, nullptr, 1);
+    RTE_TRY(gemm_f64(h->stream, rows, d.nSm, d.dM, tmp, d.dM, d.WmNT, d.nSm, X, d.nSm, 1.0, 1.0, 0,
+                     nullptr, nullptr, nullptr, 1));
     return RTE_OK;
 }
 
@@ -1056,8 +1056,8 @@ int mk_prec(rte_handle* h, const double* B, double* X, double* tmp, int nrhs) {
 int mk_apply(rte_handle* h, const double* Z, double* Y, double* G, int nrhs) {
     const DevSystem& d = h->d;
     Scope sc(h, "mk_apply");
-    gemm_f64(h->stream, nrhs * d.nRm, d.nSm, d.nSm, Z, d.nSm, d.Sm, d.nSm, G, d.nSm, 1.0, 0.0,
-             0, nullptr, nullptr, nullptr, 1);
+    RTE_TRY(gemm_f64(h->stream, nrhs * d.nRm, d.nSm, d.nSm, Z, d.nSm, d.Sm, d.nSm, G, d.nSm, 1.0, 0.0,
+                     0, nullptr, nullptr, nullptr, 1));
     mk_combine(h->stream, d, Z, G, Y, nrhs);
     return RTE_OK;
 }
@@ -1265,8 +1265,8 @@ int apply_E(rte_handle* h, const double* x, double* y, int nrhs, bool with_k,
                                d.nSp, S, V, d.nSp, 0, nullptr, 1, d.split_S));
         } else {
             Scope sc(h, "gemm_kplus");
-            gemm_f64(h->stream, nrhs * d.nRp, d.nSp, d.nSp, x, d.nSp, d.Sp, d.nSp, V, d.nSp, 1.0,
-                     0.0, 0, nullptr, nullptr, nullptr, 1);
+            RTE_TRY(gemm_f64(h->stream, nrhs * d.nRp, d.nSp, d.nSp, x, d.nSp, d.Sp, d.nSp, V, d.nSp, 1.0,
+                             0.0, 0, nullptr, nullptr, nullptr, 1));
         }
     }
     Scope sc(h, "apply_even");
@@ -1518,8 +1518,8 @@ int restrict_(rte_handle* h, const double* x, double* qc, int nrhs, const float*
     Scope sc(h, "restrict");
     if (!restrict_rows(h->stream, nrhs * d.nRp, d.nSp, d.dP, x, d.WpN, h->mixed ? d.lo.WpN : nullptr,
                        qc, sub))
-        gemm_f64(h->stream, nrhs * d.nRp, d.dP, d.nSp, x, d.nSp, d.WpN, d.dP, qc, d.dP, 1.0, 0.0,
-                 0, nullptr, nullptr, nullptr, 1);
+        RTE_TRY(gemm_f64(h->stream, nrhs * d.nRp, d.dP, d.nSp, x, d.nSp, d.WpN, d.dP, qc, d.dP, 1.0, 0.0,
+                         0, nullptr, nullptr, nullptr, 1));
     return RTE_OK;
 }
 
@@ -1528,8 +1528,8 @@ int prolong_add(rte_handle* h, const double* uc, double* x, int nrhs, double bet
     Scope sc(h, "prolong");
     if (!prolong_rows(h->stream, nrhs * d.nRp, d.nSp, d.dP, uc, d.WpNT,
                       h->mixed ? d.lo.WpNT : nullptr, x, beta))
-        gemm_f64(h->stream, nrhs * d.nRp, d.nSp, d.dP, uc, d.dP, d.WpNT, d.nSp, x, d.nSp, 1.0,
-                 beta, 0, nullptr, nullptr, nullptr, 1);
+        RTE_TRY(gemm_f64(h->stream, nrhs * d.nRp, d.nSp, d.dP, uc, d.dP, d.WpNT, d.nSp, x, d.nSp, 1.0,
+                         beta, 0, nullptr, nullptr, nullptr, 1));
     return RTE_OK;
 }
 
@@ -2207,8 +2207,8 @@ int rte_operator(rte_handle* h, int op, const double* in, double* out, int nrhs)
         case RTE_OP_A: apply_A(s, d, in, out, nrhs); break;
         case RTE_OP_AT: apply_even(s, d, in, nullptr, nullptr, out, nrhs, 1); break;
         case RTE_OP_KPLUS:
-            gemm_f64(s, nrhs * d.nRp, d.nSp, d.nSp, in, d.nSp, d.Sp, d.nSp, h->e8, d.nSp, 1.0,
-                     0.0, 0, nullptr, nullptr, nullptr, 1);
+            RTE_TRY(gemm_f64(s, nrhs * d.nRp, d.nSp, d.nSp, in, d.nSp, d.Sp, d.nSp, h->e8, d.nSp, 1.0,
+                             0.0, 0, nullptr, nullptr, nullptr, 1));
             apply_even(s, d, nullptr, h->e8, h->e8, out, nrhs, 4);
             k_neg<<<(unsigned)((nrhs * (size_t)d.nRp * d.nSp + 255) / 256), 256, 0, s>>>(
                 out, (size_t)nrhs * d.nRp * d.nSp);
