@@ -1343,6 +1343,8 @@ int read_status(rte_handle* h, SolveStatus& st) {
 // a relative residual of at least this (the FP64 outer loop absorbs it).
 constexpr double kLowInnerTol = 1e-5;
 
+// x = E_0^{-1} b.  Uses e5 and e6 where b or x is not aligned for the FP32
+// multigrid route.
 int e0_inv(rte_handle* h, const double* b, double* x, int nrhs) {
     if (h->d.e0_direct) {
         {
@@ -1355,15 +1357,25 @@ int e0_inv(rte_handle* h, const double* b, double* x, int nrhs) {
         h->e0_active_vcycles += 1.0;
         return RTE_OK;
     }
+    // the FP32 kernel reads b and writes x 16 bytes at a time: a caller's
+    // vector that is not aligned for that goes through an array of the handle
+    const size_t bytes = sizeof(double) * nrhs * h->d.nRp * h->d.nSp;
+    double* out = x;
     if (h->mixed) {
+        if (reinterpret_cast<uintptr_t>(b) & 15) {
+            RTE_CUDA_TRY(cudaMemcpyAsync(h->e5, b, bytes, cudaMemcpyDeviceToDevice, h->stream));
+            b = h->e5;
+        }
+        if (reinterpret_cast<uintptr_t>(x) & 15) out = h->e6;
         Scope sc(h, "e0_cg_lo");
-        RTE_TRY(e0_cg_lo(h->stream, h->d, b, x, nrhs, std::max(h->opt.e0_tol, kLowInnerTol),
+        RTE_TRY(e0_cg_lo(h->stream, h->d, b, out, nrhs, std::max(h->opt.e0_tol, kLowInnerTol),
                          h->opt.e0_maxit, h->e0work, h->e0bytes, h->status));
     } else {
         Scope sc(h, "e0_cg");
         RTE_TRY(e0_cg(h->stream, h->d, b, x, nrhs, h->opt.e0_tol, h->opt.e0_maxit, h->e0work,
                       h->e0bytes, h->status));
     }
+    if (out != x) RTE_CUDA_TRY(cudaMemcpyAsync(x, out, bytes, cudaMemcpyDeviceToDevice, h->stream));
     SolveStatus st;
     RTE_TRY(read_status(h, st));
     h->e0_iters = st.iterations;
@@ -1461,12 +1473,6 @@ int apply_P1_pcg_lo(rte_handle* h, const double* b, double* z, int nrhs) {
     cudaStream_t s = h->stream;
     double *R = h->e9, *P = h->e10, *Y = h->e6;
     double *rho = h->sc + 8 * n, *alpha = h->sc + 10 * n, *beta = h->sc + 11 * n;
-    // the multigrid route reads its right-hand side 16 bytes at a time: a
-    // caller's vector that is not aligned for that is copied first
-    if (!d.e0_direct && (reinterpret_cast<uintptr_t>(b) & 15)) {
-        RTE_CUDA_TRY(cudaMemcpyAsync(R, b, sizeof(double) * n * len, cudaMemcpyDeviceToDevice, s));
-        b = R;
-    }
     RTE_TRY(e0_inv(h, b, Y, n));                       // y = E_0^{-1} b
     {
         Scope sc(h, "axpy");

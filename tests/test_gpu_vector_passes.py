@@ -89,3 +89,26 @@ def test_p1_in_place():
         assert (got - want).abs().max().item() <= 1e-7 * want.abs().max().item()
     finally:
         s.close()
+
+
+@pytest.mark.parametrize('precision', [1, 2])
+def test_unaligned_vectors_on_the_multigrid_route_of_p1_l(precision):
+    # P_1^l hands the caller's vectors to E_0^{-1} themselves, as the operator
+    # alone does; E_0 CG to 1e-5, the bound of the test above
+    import paper_2102_09038_gb300 as rte
+    m, levels, nrhs = 9, 2, 2
+    p = workloads.constant(m, levels, 0.6, 1.5, 1.2)
+    s = rte.Solver(p, n_plus=2, n_minus=3, precision=precision, max_rhs=nrhs, l=2,
+                   p1_route=rte.P1_RICHARDSON, e0_route=rte.E0_MULTIGRID, e0_tol=1e-5)
+    try:
+        x = np.random.default_rng(m).standard_normal((nrhs, (m + 1) ** 2, 4 << (2 * levels)))
+        for call in (lambda a, o: s.precond(a, False, o), lambda a, o: s.operator('E0_INV', a, o)):
+            got = []
+            for by_in, by_out in ((0, 0), (1, 0), (0, 1), (1, 1)):
+                out = shifted(np.zeros_like(x), by_out)
+                call(shifted(x, by_in), out)
+                got.append(out.cpu().numpy())
+            for g in got[1:]:
+                assert np.abs(g - got[0]).max() <= 1e-4 * np.abs(got[0]).max()
+    finally:
+        s.close()
