@@ -414,7 +414,11 @@ long long rte_kernel_launches(void);
  * E_0 / E_c kernels, and an mbarrier wait of the tensor-core pipelines.  A
  * wait that runs out makes the kernel record the failure and return; the
  * calling function then returns RTE_ERR_TIMEOUT and the CUDA context stays
- * usable.  rte_set_wait_limit sets the limit (seconds, in (0, 60]; default
+ * usable.  rte_apply, rte_precond without P_2 and the rte_operator steps that
+ * only queue work do not wait for it: a wait of the tensor-core pipelines or
+ * of the E_0 sweeps that runs out in them is reported by the next call on the
+ * device that synchronises (rte_solve, rte_odd, rte_rates, rte_precond with
+ * P_2, the GEMM entry points).  rte_set_wait_limit sets the limit (seconds, in (0, 60]; default
  * 2 s): for grid barriers of every launch made after the call, for mbarrier
  * waits on the current device.  Not thread-safe against concurrent
  * launches. */
@@ -430,6 +434,12 @@ int rte_set_wait_limit(double seconds);
  * out, else RTE_OK. */
 int rte_barrier_selftest(int blocks, int skip_block, int rounds, void* stream, int* timed_out,
                          int* passed_blocks);
+
+/* Self-test of the tensor-core pipelines' bounded wait: one wait for an
+ * arrival that never comes, queued on `stream` and synchronised.  It runs out
+ * after the current limit and leaves the device's flag set, for the next call
+ * that reads it to report.  Returns RTE_OK. */
+int rte_pipeline_selftest(void* stream);
 
 void rte_destroy(rte_handle* h);
 

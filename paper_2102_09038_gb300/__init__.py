@@ -91,7 +91,7 @@ EXPORTED = ['rte_default_options', 'rte_setup', 'rte_sizes', 'rte_rhs', 'rte_inf
             'rte_kernel_launches', 'rte_gemm_lowp', 'rte_dgemm_split',
             'rte_trace_enable', 'rte_estimate_bytes', 'rte_server_create',
             'rte_server_submit', 'rte_server_wait', 'rte_server_destroy', 'rte_solve_batch',
-            'rte_trace_read', 'rte_destroy', 'rte_set_wait_limit', 'rte_barrier_selftest',
+            'rte_trace_read', 'rte_destroy', 'rte_set_wait_limit', 'rte_barrier_selftest', 'rte_pipeline_selftest',
             'rte_set_stream', 'rte_server_cache_stats',
             'rte_h2_default_options', 'rte_h2_create', 'rte_h2_apply', 'rte_h2_get_info',
             'rte_h2_dense', 'rte_h2_destroy', 'rte_h2_plan_info',
@@ -153,6 +153,7 @@ def load(path=LIB_PATH):
     lib.rte_trace_read.argtypes = [P, ctypes.POINTER(D), I, ctypes.POINTER(I)]
     lib.rte_set_wait_limit.argtypes = [D]
     lib.rte_barrier_selftest.argtypes = [I, I, I, P, ctypes.POINTER(I), ctypes.POINTER(I)]
+    lib.rte_pipeline_selftest.argtypes = [P]
     lib.rte_kernel_launches.argtypes = []
     lib.rte_kernel_launches.restype = ctypes.c_longlong
     lib.rte_destroy.argtypes = [P]
@@ -198,6 +199,15 @@ def barrier_selftest(blocks, skip_block=-1, rounds=4, stream=None):
     if rc not in (0, 5):
         _check(rc)
     return rc, to.value, ok.value
+
+
+def pipeline_selftest(stream=None):
+    """One wait of the tensor-core pipelines that runs out after the current
+    limit; the next call that reads the device's flag reports it."""
+    import torch
+    lib = load()
+    st = stream if stream is not None else torch.cuda.current_stream()
+    _check(lib.rte_pipeline_selftest(ctypes.c_void_p(st.cuda_stream)))
 
 
 def gemm_lowp(A, Bt, out_bf16=False, stream=None):

@@ -70,10 +70,11 @@ struct rte_handle {
     float* zf = nullptr;
     double *partial = nullptr, *sc = nullptr;                               // reductions
     // pinned host memory of the outer iteration's one synchronisation: the
-    // residual sums, the coarse solve's status, the E_0 sweeps' flag
+    // residual sums, the coarse solve's status, the flags of the E_0 sweeps'
+    // and of the tensor-core pipelines' waits
     double* host_sums = nullptr;
     SolveStatus* host_status = nullptr;
-    int* host_e0_error = nullptr;
+    int *host_e0_error = nullptr, *host_tc_error = nullptr;
     void* e0work = nullptr;
     size_t e0bytes = 0;
     void* cowork = nullptr;
@@ -899,12 +900,13 @@ int alloc_workspace(rte_handle* h, int nrhs) {
     RTE_TRY(dalloc(h, &h->c2, nc));
     RTE_TRY(dalloc(h, &h->partial, (size_t)nrhs * 3 * 1024));
     char* pin = nullptr;
-    if (cudaMallocHost(&pin, (size_t)nrhs * 3 * sizeof(double) + sizeof(SolveStatus) + sizeof(int)) != cudaSuccess)
+    if (cudaMallocHost(&pin, (size_t)nrhs * 3 * sizeof(double) + sizeof(SolveStatus) + 2 * sizeof(int)) != cudaSuccess)
         return fail(RTE_ERR_NOMEM, "pinned iteration state");
     h->host_sums = reinterpret_cast<double*>(pin);
     h->host_status = reinterpret_cast<SolveStatus*>(h->host_sums + (size_t)nrhs * 3);
     h->host_e0_error = reinterpret_cast<int*>(h->host_status + 1);
-    *h->host_e0_error = 0;
+    h->host_tc_error = h->host_e0_error + 1;
+    *h->host_e0_error = *h->host_tc_error = 0;
     RTE_TRY(dalloc(h, &h->sc, (size_t)nrhs * 16));
     char* w = nullptr;
     if (!d.e0_direct) {
@@ -1339,6 +1341,22 @@ int read_status(rte_handle* h, SolveStatus& st) {
     return RTE_OK;
 }
 
+// Whether a wait ran out in the E_0 sweeps or the tensor-core products queued
+// so far: the flags' copies, queued before a synchronisation of the caller's,
+// and their check after it (a flag that was set is cleared).
+int flags_fetch(rte_handle* h) {
+    if (h->d.e0_direct) RTE_TRY(e0_direct_error_fetch(h->stream, h->host_e0_error));
+    if (h->mixed || h->d.split_S > 0) RTE_TRY(tc_gemm_error_fetch(h->stream, h->host_tc_error));
+    return RTE_OK;
+}
+
+int flags_check(rte_handle* h) {
+    const int e0 = e0_direct_error_check(h->stream, *h->host_e0_error);
+    const int tc = tc_gemm_error_check(h->stream, *h->host_tc_error);
+    *h->host_e0_error = *h->host_tc_error = 0;
+    return e0 != RTE_OK ? e0 : tc;
+}
+
 // FP32 CG stalls near its rounding level: mixed modes stop the E_0 solves at
 // a relative residual of at least this (the FP64 outer loop absorbs it).
 constexpr double kLowInnerTol = 1e-5;
@@ -1572,7 +1590,10 @@ int precond(rte_handle* h, const double* r, double* s, int nrhs, bool p2) {
     RTE_TRY(precond_queue(h, r, s, nrhs, p2));
     if (!p2) return RTE_OK;
     SolveStatus st;
-    RTE_TRY(read_status(h, st));
+    RTE_TRY(flags_fetch(h));
+    const int rc = read_status(h, st);
+    RTE_TRY(flags_check(h));
+    RTE_TRY(rc);
     h->co_iters = st.iterations;
     // s <- s - W u_c, so that u_{n+1} = u_n - s = u_{n+1/2} + W u_c
     RTE_TRY(prolong_add(h, h->c2, s, nrhs, 1.0));
@@ -2413,9 +2434,10 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
         if (it > 0 && p2)
             RTE_CUDA_TRY(cudaMemcpyAsync(h->host_status, h->status, sizeof(SolveStatus),
                                          cudaMemcpyDeviceToHost, s));
-        if (it > 0 && d.e0_direct) RTE_TRY(e0_direct_error_fetch(s, h->host_e0_error));
+        RTE_TRY(flags_fetch(h));
         RTE_CUDA_TRY(cudaStreamSynchronize(s));
         settle_mk(h);
+        RTE_TRY(flags_check(h));
         if (it > 0 && p2) {
             if (h->host_status->timed_out) return fail(RTE_ERR_TIMEOUT, "a bounded grid barrier timed out");
             h->co_iters = h->host_status->iterations;
@@ -2431,7 +2453,6 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
             if (it > 0) energy = std::max(energy, std::sqrt(std::max(0.0, hd1[k] - hd2[k])));
         }
         if (stats && stats->history && it < stats->history_cap) stats->history[it] = worst;
-        if (it > 0 && d.e0_direct) RTE_TRY(e0_direct_error_check(s, *h->host_e0_error));
         if (nan) { rc = fail(RTE_ERR_DIVERGED, "residual is NaN or Inf"); break; }
         if (worst <= tol) break;
         if (it >= h->opt.max_iter) { rc = fail(RTE_ERR_MAXITER, "outer iteration cap reached"); break; }
@@ -2605,6 +2626,8 @@ int rte_gemm_lowp(const void* A, const void* Bt, void* C, int M, int N, int K, i
     RTE_TRY(tc_gemm((cudaStream_t)stream, g));
     return tc_gemm_error((cudaStream_t)stream);
 }
+
+int rte_pipeline_selftest(void* stream) { return tc_wait_selftest((cudaStream_t)stream); }
 
 void rte_destroy(rte_handle* h) {
     if (!h) return;

@@ -226,6 +226,15 @@ k_tc_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUte
                      "r"(kTmemCols));
 }
 
+// A wait for an arrival that never comes: it runs out and sets the pipelines'
+// flag, as a wait in the kernels above would.
+__global__ void k_wait_alone() {
+    __shared__ __align__(8) uint64_t bar;
+    if (threadIdx.x != 0) return;
+    mbar_init(smem_u32(&bar), 1);
+    mbar_wait(smem_u32(&bar), 0);
+}
+
 template <int BN>
 constexpr size_t smem_bytes() {
     return 1024 + (size_t)kStages * (kBM + BN) * kRowBytes;   // 1024: alignment
@@ -270,16 +279,31 @@ int tc_set_wait_cycles(long long cycles) {
     return RTE_OK;
 }
 
+int tc_gemm_error_fetch(cudaStream_t s, int* host) {
+    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(host, g_tc_error, sizeof(int), 0,
+                                           cudaMemcpyDeviceToHost, s));
+    return RTE_OK;
+}
+
+int tc_gemm_error_check(cudaStream_t s, int flag) {
+    if (!flag) return RTE_OK;
+    const int zero = 0;
+    cudaMemcpyToSymbolAsync(g_tc_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
+    return fail(RTE_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
+}
+
 int tc_gemm_error(cudaStream_t s) {
     int e = 0;
-    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(&e, g_tc_error, sizeof(int), 0,
-                                           cudaMemcpyDeviceToHost, s));
+    RTE_TRY(tc_gemm_error_fetch(s, &e));
     RTE_CUDA_TRY(cudaStreamSynchronize(s));
-    if (e) {
-        const int zero = 0;
-        cudaMemcpyToSymbolAsync(g_tc_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
-        return fail(RTE_ERR_TIMEOUT, "a tensor-core GEMM pipeline wait timed out");
-    }
+    return tc_gemm_error_check(s, e);
+}
+
+int tc_wait_selftest(cudaStream_t s) {
+    count_launches(1);
+    k_wait_alone<<<1, 32, 0, s>>>();
+    RTE_CUDA_TRY(cudaGetLastError());
+    RTE_CUDA_TRY(cudaStreamSynchronize(s));
     return RTE_OK;
 }
 

@@ -121,3 +121,26 @@ def test_barrier_wait_runs_out_and_context_stays_usable():
     rc, timed_out, passed = rte.barrier_selftest(152, skip_block=-1, rounds=16)
     assert (rc, timed_out, passed) == (0, 0, 152)
     solve_ok(rte.Solver(small(), n_plus=2, n_minus=3), small())
+
+
+@pytest.mark.parametrize('prec, kw', [(1, {}), (2, {}), (0, {'dgemm': 2})])
+def test_pipeline_wait_that_ran_out_is_reported(prec, kw):
+    # the tensor-core pipelines' flag, set by a wait that runs out after 1 ms:
+    # the next solve, preconditioner step or odd part reports it, once, and
+    # the handle then solves normally; an apply alone only queues its work
+    import paper_2102_09038_gb300 as rte
+    p = small()
+    s = rte.Solver(p, n_plus=2, n_minus=3, precision=prec, **kw)
+    q = s.rhs(torch.tensor(p.q_nodal, dtype=torch.float64, device='cuda'))
+    for call in (lambda: s.solve(q, tol=1e-8), lambda: s.precond(q, True), lambda: s.odd(q)):
+        rte.set_wait_limit(1e-3)
+        try:
+            rte.pipeline_selftest()
+        finally:
+            rte.set_wait_limit(2.0)
+        s.apply(q)
+        with pytest.raises(rte.RteError) as e:
+            call()
+        assert e.value.code == 5   # RTE_ERR_TIMEOUT
+        solve_ok(s, p)
+    s.close()
