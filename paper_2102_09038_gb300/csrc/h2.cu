@@ -408,9 +408,10 @@ k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict_
 // block of 128 threads per (128-row tile, group of G output blocks): warp 0
 // lane 0 loads the A tile (128 rows x 64 columns of In, one 128-byte swizzled
 // row per matrix row) and the B tiles of the outputs that take this input
-// (64 x 64 matrices, stored K-major as Bt[output][input]) by TMA into a
-// 4-stage ring, warp 1 issues the MMAs, and the four warps drain 64 columns of
-// the accumulator per output.  Every wait is bounded (tc::mbar_wait).
+// (64 x 64 matrices, stored K-major as Bt[output][input]) by TMA into a ring
+// of 4 stages (3 for pairs), warp 1 issues the MMAs, and the four warps drain
+// 64 columns of the accumulator per output.  Every wait is bounded
+// (tc::mbar_wait).
 //
 // What bounds it: with G = 1 the reads from L2 (16 KB of A and 8 KB of B for
 // one 128 x 64 x 64 product; 80 % of L2's rate) and MMAs 64 columns wide (a
@@ -723,9 +724,9 @@ int run_tc(cudaStream_t s, const TcList& T, int rows, const void* In, long long 
     // 1203, 512 rows (664 groups) 374 against 389, 256 rows (332) 264 against
     // 251; of 4096 directions, 1024 rows (304) 191 against 187)
     const int rtiles = (rows + kTcRows - 1) / kTcRows;
-    const bool group = T.group.nout > 0 && (long long)T.group.nout * rtiles >= 4 * device_sm_count();
-    return group ? launch_tc<kTcGroup>(s, ma, mb, T.group, rows, Old, Out, ldo)
-                 : launch_tc<1>(s, ma, mb, T.one, rows, Old, Out, ldo);
+    return h2_takes_groups(T.group.nout, rtiles, device_sm_count())
+               ? launch_tc<kTcGroup>(s, ma, mb, T.group, rows, Old, Out, ldo)
+               : launch_tc<1>(s, ma, mb, T.one, rows, Old, Out, ldo);
 }
 
 template <typename T, int kMode, bool kAccum, int TM, int TN>
@@ -937,10 +938,7 @@ int build_tc(rte_h2* h, int q, const rte::H2Lists& lists, cudaStream_t s) {
             c.mat[e] = (int)(base + (from < 0 ? (long long)e : c.mat[e] - from));
         RTE_TRY(upload_list(h, c, d.one, s));
         const H2List g = h2_group_list(c, kTcGroup);
-        // tiles read by groups (a 16 KB input, 8 KB matrices) against singly
-        // where blocks have entries enough to hide their ends
-        if (2 * g.in_blk.size() + c.in_blk.size() < 0.8 * 3 * c.in_blk.size() &&
-            g.in_blk.size() >= 8 * g.ptr.size()) {
+        if (h2_group_pays(c, g)) {
             RTE_TRY(upload_list(h, g, d.group, s));
             d.group.nout /= kTcGroup;
         }

@@ -73,6 +73,14 @@ void h2_lists(const H2Plan& P, const H2Pool& pool, H2Lists& L);
 // entry's input.  Every output meets its entries in the list's order.  Empty
 // when an output has no entries.
 H2List h2_group_list(const H2List& l, int G);
+// Whether a list's groups save enough: the tiles read by groups (a 16 KB input
+// and its 8 KB matrices) against singly, where blocks have entries enough to
+// hide their ends.
+bool h2_group_pays(const H2List& l, const H2List& grouped);
+// Whether a call takes the groups: every SM gets two blocks twice over.
+inline bool h2_takes_groups(int groups, int row_tiles, int sms) {
+    return groups > 0 && (long long)groups * row_tiles >= 4 * sms;
+}
 
 // Limit of one mbarrier wait of the tensor-core H^2 products (SM cycles).
 int h2_set_wait_cycles(long long cycles);

@@ -259,4 +259,9 @@ H2List h2_group_list(const H2List& l, int G) {
     return g;
 }
 
+bool h2_group_pays(const H2List& l, const H2List& g) {
+    const size_t one = l.in_blk.size(), both = g.in_blk.size();
+    return both > 0 && 2 * both + one < 0.8 * 3 * one && both >= 8 * g.ptr.size();
+}
+
 }  // namespace rte
