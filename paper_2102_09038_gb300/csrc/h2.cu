@@ -259,12 +259,14 @@ __device__ __forceinline__ double hg_t(double mu, double g, double c0) {
 // have no tile at all (S^- of 1024 directions, 130 rows: 48 to 144 tiles of
 // 64 x 64 a stage).  bsr_tile takes the tile with the least work on the
 // busiest SM; A is read four values of k at a time, which takes the products
-// from shared memory's rate to the FP32 units'.  Measured, 130 rows of S^- on
-// 1024 directions, FP32: an apply 231 -> 169 us
-// (couplings 29 us, 65 before an entry's indices were read a chunk ahead of
-// its loads; near field 106).
-template <typename T, int kMode, bool kAccum, int TM, int TN>
-__global__ void __launch_bounds__(256)
+// from shared memory's rate to the FP32 units'.  kAhead: the next chunk's loads
+// run under the current one's products (97 registers at 64 x 64, two blocks an
+// SM in FP32); without it three blocks an SM hide each other's loads.  Measured,
+// 130 rows of S^- on 1024 directions, FP32: an apply 231 -> 169 us (couplings
+// 29 us, 65 before an entry's indices were read a chunk ahead of its loads;
+// near field 106); 3000 rows of S^+ on 16384: 28.1 -> 27.4 ms.
+template <typename T, int kMode, bool kAccum, int TM, int TN, bool kAhead>
+__global__ void __launch_bounds__(256, kAhead ? 0 : 3)
 k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict__ In,
          long long ldi, T* __restrict__ Out, long long ldo, const int* __restrict__ out_blk,
          const int* __restrict__ ptr, const int* __restrict__ in_blk, const int* __restrict__ mat,
@@ -336,8 +338,9 @@ k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict_
             }
         }
     };
-    if (chunks > 0) load(0);
+    if (kAhead && chunks > 0) load(0);
     for (int c = 0; c < chunks; ++c) {
+        if (!kAhead) load(c);
         __syncthreads();   // the chunk before has been read
 #pragma unroll
         for (int s = 0; s < RM; ++s) {
@@ -373,7 +376,7 @@ k_h2_bsr(int rows, int rtiles, int nout, int k, int parity, const T* __restrict_
             }
         }
         __syncthreads();
-        if (c + 1 < chunks) load(c + 1);
+        if (kAhead && c + 1 < chunks) load(c + 1);
 #pragma unroll 4
         for (int k0 = 0; k0 < KC; k0 += VN) {
             V a[RM];
@@ -729,14 +732,14 @@ int run_tc(cudaStream_t s, const TcList& T, int rows, const void* In, long long 
                : launch_tc<1>(s, ma, mb, T.one, rows, Old, Out, ldo);
 }
 
-template <typename T, int kMode, bool kAccum, int TM, int TN>
+template <typename T, int kMode, bool kAccum, int TM, int TN, bool kAhead = true>
 int run_tile(cudaStream_t s, const DevList& L, int rows, int k, int parity, const T* In,
              long long ldi, T* Out, long long ldo, const T* pool, const T* xi, double g) {
     const int rtiles = (rows + TM - 1) / TM;
     const long long grid = (long long)((L.nout + kGroup - 1) / kGroup) * kGroup * rtiles * (kH2B / TN);
     if (grid > 0x7fffffffLL) return fail(RTE_ERR_ARG, "H2 apply: too many rows for one launch");
     const T c0 = T((1.0 - g * g) / (4.0 * kPi));
-    k_h2_bsr<T, kMode, kAccum, TM, TN><<<(unsigned)grid, 256, 0, s>>>(
+    k_h2_bsr<T, kMode, kAccum, TM, TN, kAhead><<<(unsigned)grid, 256, 0, s>>>(
         rows, rtiles, L.nout, k, parity, In, ldi, Out, ldo, L.out_blk, L.ptr, L.in_blk, L.mat, pool,
         xi, T(g), c0);
     count_launches(1);
@@ -744,26 +747,40 @@ int run_tile(cudaStream_t s, const DevList& L, int rows, int k, int parity, cons
 }
 
 // The tile of a call: TM = 64 or 32 rows, TN = 64 or 32 columns, whichever
-// gives the busiest SM the least work.  A tile's clocks per step of k, from
-// the FP32 units' rate (64 x 64: 32, 64 x 32: 16) or, below 64 rows, shared
-// memory's (20 and 12); in FP64 the units' two multiply-adds a clock; plus
-// the evaluation of a coupling matrix' TN entries per step.  Every column (or
-// row) tile more re-reads A (or B): a tenth on top, so that calls with many
-// tiles stay at 64 x 64.
+// gives the busiest SM the least work, a tile's clocks per step of k times the
+// tiles of that SM.  In FP32 the clocks are the ratios of calls with many tiles
+// an SM (S^+ of 4096 directions, 3000 rows: 64 x 64 5.61 ms an apply, 64 x 32
+// 6.66, 32 x 64 7.82, 32 x 32 9.18), plus a quarter for each of a coupling
+// matrix' TN entries per step; in FP64 the units' two multiply-adds a clock,
+// the 30 clocks of a coupling matrix' entry, and a tenth for re-reading A or B.
+// Both sides of the line, FP32: 130 rows of S^- of 256 directions 59.5, 50.5,
+// 49.2, 40.8 us (64 x 64, 32 x 64, 64 x 32, 32 x 32; takes the last), 700 rows
+// of S^- of 1024 474, 634, 547, 673 (takes the first).
+// Tile 4 is 64 x 64 with three blocks an SM that load a chunk only when the one
+// before has been used: better where all blocks run at once (more than two an
+// SM, up to three) or many follow each other (more than four): 3000 rows of
+// S^+ of 16384 directions 27.4 against 29.7 ms, 300 rows of 4096 875 against
+// 952 us.  Between, and below, the two blocks that load ahead are (1500 rows of
+// S^- of 256 directions, 1.9 blocks an SM: 94 against 119 us; 450 rows of S^+
+// of 4096, 3.4: 1210 against 1260).
 template <typename T>
 int bsr_tile(int nout, int rows, bool couple) {
     const double sms = device_sm_count();
+    constexpr double f32_step[4] = {32.0, 22.3, 19.0, 13.1};
     int best = 0;
     double cost = 1e300;
     for (int t = 0; t < 4; ++t) {
         const int TM = t & 1 ? 32 : 64, TN = t & 2 ? 32 : 64;
-        double step = sizeof(T) == 8 ? TM * TN / 2 : TM == 64 ? TN / 2 : TN == 64 ? 20 : 12;
+        double step = sizeof(T) == 8 ? TM * TN / 2 : f32_step[t];
         if (couple) step += (sizeof(T) == 8 ? 30 : 0.25) * TN;
+        if (sizeof(T) == 8 && t) step *= 1.1;
         const double blocks = (double)nout * ((rows + TM - 1) / TM) * (kH2B / TN);
-        const double c = std::ceil(blocks / sms) * step * (t ? 1.1 : 1.0);
+        const bool three = sizeof(T) == 4 && t == 0 &&
+                           ((blocks > 2 * sms && blocks <= 3 * sms) || blocks > 4 * sms);
+        const double c = std::ceil(blocks / sms) * step * (three ? 0.92 : 1.0);
         if (c < cost) {
             cost = c;
-            best = t;
+            best = three ? 4 : t;
         }
     }
     return best;
@@ -776,7 +793,12 @@ int run_list(cudaStream_t s, const DevList& L, int rows, Args... args) {
         case 0: return run_tile<T, kMode, kAccum, 64, 64>(s, L, rows, args...);
         case 1: return run_tile<T, kMode, kAccum, 32, 64>(s, L, rows, args...);
         case 2: return run_tile<T, kMode, kAccum, 64, 32>(s, L, rows, args...);
-        default: return run_tile<T, kMode, kAccum, 32, 32>(s, L, rows, args...);
+        case 3: return run_tile<T, kMode, kAccum, 32, 32>(s, L, rows, args...);
+        default:   // FP32 only
+            if constexpr (sizeof(T) == 4)
+                return run_tile<T, kMode, kAccum, 64, 64, false>(s, L, rows, args...);
+            else
+                return run_tile<T, kMode, kAccum, 64, 64>(s, L, rows, args...);
     }
 }
 
