@@ -121,6 +121,18 @@ struct SolveStatus {
     long long active_quads;   // E_0 quad kernel: active quads summed over its V-cycles
 };
 
+// What the host reads at the outer iteration's synchronisation beside the
+// residual sums: the coarse solve's status, and whether a wait ran out in the
+// E_0 sweeps or the tensor-core pipelines (copies of their device flags).
+struct IterState {
+    SolveStatus status;
+    int e0_flag, tc_flag;
+};
+struct IterStateSrc {          // device pointers
+    const SolveStatus* status;
+    const int *e0_flag, *tc_flag;
+};
+
 // ------------------------------------------------------------- launchers
 // C = alpha * op(A B) + beta * C for row-major A (M x K), B (K x N),
 // C (M x N); epi selects a per-element factor applied to A B:
@@ -184,9 +196,12 @@ void p1_step(cudaStream_t s, const double* alpha, bool first, bool last, const d
 // beta = R.Y / rho, rho = R.Y, P = Y + beta P, F = (float)P
 void p1_direction(cudaStream_t s, const double* R, const double* Y, double* P, float* F, size_t len,
                   int nrhs, double* partial, double* rho, double* beta);
-// out = [R.R] and, with D, [D.R], [D.Rp], nrhs values each
+// out = [R.R], [D.R], [D.Rp], nrhs values each (the last two only with D), and
+// *state = the state src points at
 void residual_sums(cudaStream_t s, const double* R, const double* D, const double* Rp, size_t len,
-                   int nrhs, double* partial, double* out);
+                   int nrhs, double* partial, double* out, const IterStateSrc& src, IterState* state);
+// *state = the state src points at
+void gather_state(cudaStream_t s, const IterStateSrc& src, IterState* state);
 // U -= S, D = -S
 void update_solution(cudaStream_t s, const double* S, double* U, double* D, size_t n);
 void convert(cudaStream_t s, const float* x, double* y, size_t n);
@@ -247,9 +262,9 @@ int e0_direct_solve(cudaStream_t s, const DevSystem& d, const double* B, double*
                     bool fp64);
 // Reads and clears the flag a timed-out factor-block wait sets (synchronises s).
 int e0_direct_error(cudaStream_t s);
-// The same in two halves around a synchronisation of the caller's: the copy
-// of the flag to (pinned) host memory, and its check afterwards.
-int e0_direct_error_fetch(cudaStream_t s, int* host);
+// The flag's address on the current device, and the check (and clearing) of a
+// copy the caller has read.
+int e0_direct_flag(const int** flag);
 int e0_direct_error_check(cudaStream_t s, int flag);
 // Limit of one such wait on the current device (SM clock cycles).
 int e0_set_wait_cycles(long long cycles);

@@ -669,8 +669,8 @@ int e0_direct_solve(cudaStream_t s, const DevSystem& d, const double* B, double*
     return solve<float>(s, d, d.e0lu32, B, X, nrhs);
 }
 
-int e0_direct_error_fetch(cudaStream_t s, int* host) {
-    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(host, g_e0_error, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
+int e0_direct_flag(const int** flag) {
+    RTE_CUDA_TRY(cudaGetSymbolAddress((void**)flag, g_e0_error));
     return RTE_OK;
 }
 
@@ -683,7 +683,7 @@ int e0_direct_error_check(cudaStream_t s, int flag) {
 
 int e0_direct_error(cudaStream_t s) {
     int e = 0;
-    RTE_TRY(e0_direct_error_fetch(s, &e));
+    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(&e, g_e0_error, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
     RTE_CUDA_TRY(cudaStreamSynchronize(s));
     return e0_direct_error_check(s, e);
 }

@@ -946,13 +946,23 @@ k_p1_direction(const double* __restrict__ beta, const double* __restrict__ Y, do
     }
 }
 
+__device__ void copy_state(const IterStateSrc& src, IterState* state) {
+    state->status = *src.status;
+    state->e0_flag = *src.e0_flag;
+    state->tc_flag = *src.tc_flag;
+}
+
+__global__ void k_gather_state(IterStateSrc src, IterState* state) { copy_state(src, state); }
+
 // Sum of a right-hand side's partials, and the scalar it gives: op 0: out =
 // sum; 1: out = rho / sum (a step length); 2: out = sum / rho and rho = sum (a
-// direction's factor).  blockIdx.x: sum q nrhs + r.
+// direction's factor).  blockIdx.x: sum q nrhs + r.  state set: the iteration's
+// state beside the sums, so that one copy brings both to the host.
 __global__ void __launch_bounds__(256)
 k_sum_scalar(const double* __restrict__ partial, int nb, int op, double* rho,
-             double* __restrict__ out) {
+             double* __restrict__ out, IterStateSrc src, IterState* state) {
     const int r = blockIdx.x;
+    if (state && r == 0 && threadIdx.x == 32) copy_state(src, state);
     double s = 0.0;
     for (int b = threadIdx.x; b < nb; b += 256) s += partial[(size_t)r * 1024 + b];
     s = block_sum<256>(s);
@@ -1204,7 +1214,7 @@ void p1_start(cudaStream_t s, const double* R, const double* Y, double* P, float
         k_p1_start<2><<<dim3(nb, nrhs), 256, 0, s>>>(R, Y, P, F, len, partial);
     else
         k_p1_start<1><<<dim3(nb, nrhs), 256, 0, s>>>(R, Y, P, F, len, partial);
-    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 0, nullptr, rho);
+    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 0, nullptr, rho, {}, nullptr);
 }
 
 void p1_length(cudaStream_t s, const double* P, const float* F2, size_t len, int nrhs,
@@ -1212,7 +1222,7 @@ void p1_length(cudaStream_t s, const double* P, const float* F2, size_t len, int
     const int nb = pass_blocks(len);
     count_launches(2);
     k_p1_dot<<<dim3(nb, nrhs), 256, 0, s>>>(P, F2, len, partial);
-    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 1, rho, alpha);
+    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 1, rho, alpha, {}, nullptr);
 }
 
 void p1_step(cudaStream_t s, const double* alpha, bool first, bool last, const double* P,
@@ -1230,17 +1240,22 @@ void p1_direction(cudaStream_t s, const double* R, const double* Y, double* P, f
     const int nb = pass_blocks(len);
     count_launches(3);
     k_dot_partial<double><<<dim3(nb, nrhs), 256, 0, s>>>(R, Y, len, partial);
-    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 2, rho, beta);
+    k_sum_scalar<<<nrhs, 256, 0, s>>>(partial, nb, 2, rho, beta, {}, nullptr);
     k_p1_direction<<<dim3(nb, nrhs), 256, 0, s>>>(beta, Y, P, F, len);
 }
 
 void residual_sums(cudaStream_t s, const double* R, const double* D, const double* Rp, size_t len,
-                   int nrhs, double* partial, double* out) {
+                   int nrhs, double* partial, double* out, const IterStateSrc& src, IterState* state) {
     const int nb = pass_blocks(len);
     count_launches(2);
     if (D) k_residual_sums<true><<<dim3(nb, nrhs), 256, 0, s>>>(R, D, Rp, len, partial);
     else k_residual_sums<false><<<dim3(nb, nrhs), 256, 0, s>>>(R, D, Rp, len, partial);
-    k_sum_scalar<<<(D ? 3 : 1) * nrhs, 256, 0, s>>>(partial, nb, 0, nullptr, out);
+    k_sum_scalar<<<(D ? 3 : 1) * nrhs, 256, 0, s>>>(partial, nb, 0, nullptr, out, src, state);
+}
+
+void gather_state(cudaStream_t s, const IterStateSrc& src, IterState* state) {
+    count_launches(1);
+    k_gather_state<<<1, 1, 0, s>>>(src, state);
 }
 
 void update_solution(cudaStream_t s, const double* S, double* U, double* D, size_t n) {

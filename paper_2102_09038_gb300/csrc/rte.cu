@@ -69,12 +69,12 @@ struct rte_handle {
     void *zl1 = nullptr, *zl2 = nullptr, *xl = nullptr;
     float* zf = nullptr;
     double *partial = nullptr, *sc = nullptr;                               // reductions
-    // pinned host memory of the outer iteration's one synchronisation: the
-    // residual sums, the coarse solve's status, the flags of the E_0 sweeps'
-    // and of the tensor-core pipelines' waits
-    double* host_sums = nullptr;
-    SolveStatus* host_status = nullptr;
-    int *host_e0_error = nullptr, *host_tc_error = nullptr;
+    // What the outer iteration's one synchronisation brings to the host in one
+    // copy: the sums of ||q||^2 and of the residual [3][cap_rhs], then the
+    // iteration's state.  Pageable on the host: freeing pinned memory waits for
+    // every stream of the device, and rte_destroy waits for the handle's alone.
+    char* report = nullptr;
+    std::vector<double> host_report;
     void* e0work = nullptr;
     size_t e0bytes = 0;
     void* cowork = nullptr;
@@ -899,14 +899,8 @@ int alloc_workspace(rte_handle* h, int nrhs) {
     RTE_TRY(dalloc(h, &h->c1, nc));
     RTE_TRY(dalloc(h, &h->c2, nc));
     RTE_TRY(dalloc(h, &h->partial, (size_t)nrhs * 3 * 1024));
-    char* pin = nullptr;
-    if (cudaMallocHost(&pin, (size_t)nrhs * 3 * sizeof(double) + sizeof(SolveStatus) + 2 * sizeof(int)) != cudaSuccess)
-        return fail(RTE_ERR_NOMEM, "pinned iteration state");
-    h->host_sums = reinterpret_cast<double*>(pin);
-    h->host_status = reinterpret_cast<SolveStatus*>(h->host_sums + (size_t)nrhs * 3);
-    h->host_e0_error = reinterpret_cast<int*>(h->host_status + 1);
-    h->host_tc_error = h->host_e0_error + 1;
-    *h->host_e0_error = *h->host_tc_error = 0;
+    h->host_report.assign(((size_t)nrhs * 3 * sizeof(double) + sizeof(IterState) + 7) / 8, 0.0);
+    RTE_TRY(dalloc(h, &h->report, h->host_report.size() * sizeof(double)));
     RTE_TRY(dalloc(h, &h->sc, (size_t)nrhs * 16));
     char* w = nullptr;
     if (!d.e0_direct) {
@@ -1341,19 +1335,23 @@ int read_status(rte_handle* h, SolveStatus& st) {
     return RTE_OK;
 }
 
-// Whether a wait ran out in the E_0 sweeps or the tensor-core products queued
-// so far: the flags' copies, queued before a synchronisation of the caller's,
-// and their check after it (a flag that was set is cleared).
-int flags_fetch(rte_handle* h) {
-    if (h->d.e0_direct) RTE_TRY(e0_direct_error_fetch(h->stream, h->host_e0_error));
-    if (h->mixed || h->d.split_S > 0) RTE_TRY(tc_gemm_error_fetch(h->stream, h->host_tc_error));
-    return RTE_OK;
+// Where the iteration's state lies on the device (both flags on the handle's
+// current device).
+int state_src(rte_handle* h, IterStateSrc* src) {
+    src->status = h->status;
+    RTE_TRY(e0_direct_flag(&src->e0_flag));
+    return tc_gemm_flag(&src->tc_flag);
 }
 
-int flags_check(rte_handle* h) {
-    const int e0 = e0_direct_error_check(h->stream, *h->host_e0_error);
-    const int tc = tc_gemm_error_check(h->stream, *h->host_tc_error);
-    *h->host_e0_error = *h->host_tc_error = 0;
+// Whether a wait ran out in the E_0 sweeps or the tensor-core products queued
+// so far (a flag that was set is cleared), or in the coarse solve.
+int state_check(rte_handle* h, const IterState& st, bool coarse) {
+    const int e0 = h->d.e0_direct ? e0_direct_error_check(h->stream, st.e0_flag) : RTE_OK;
+    const int tc = h->mixed || h->d.split_S > 0 ? tc_gemm_error_check(h->stream, st.tc_flag) : RTE_OK;
+    if (coarse) {
+        if (st.status.timed_out) return fail(RTE_ERR_TIMEOUT, "a bounded grid barrier timed out");
+        h->co_iters = st.status.iterations;
+    }
     return e0 != RTE_OK ? e0 : tc;
 }
 
@@ -1589,12 +1587,14 @@ int precond(rte_handle* h, const double* r, double* s, int nrhs, bool p2) {
     p2 = p2 && h->d.dP > 0;
     RTE_TRY(precond_queue(h, r, s, nrhs, p2));
     if (!p2) return RTE_OK;
-    SolveStatus st;
-    RTE_TRY(flags_fetch(h));
-    const int rc = read_status(h, st);
-    RTE_TRY(flags_check(h));
-    RTE_TRY(rc);
-    h->co_iters = st.iterations;
+    IterStateSrc src;
+    RTE_TRY(state_src(h, &src));
+    IterState st, *dev = reinterpret_cast<IterState*>(h->report);
+    gather_state(h->stream, src, dev);
+    RTE_CUDA_TRY(cudaMemcpyAsync(&st, dev, sizeof(st), cudaMemcpyDeviceToHost, h->stream));
+    RTE_CUDA_TRY(cudaStreamSynchronize(h->stream));
+    settle_mk(h);
+    RTE_TRY(state_check(h, st, true));
     // s <- s - W u_c, so that u_{n+1} = u_n - s = u_{n+1/2} + W u_c
     RTE_TRY(prolong_add(h, h->c2, s, nrhs, 1.0));
     return RTE_OK;
@@ -2413,10 +2413,14 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
     std::vector<double> hq(nrhs);
     double* sc = h->sc;
     const bool p2 = d.dP > 0;
+    IterStateSrc src;
+    RTE_TRY(state_src(h, &src));
+    double* sums = reinterpret_cast<double*>(h->report);
+    IterState* state = reinterpret_cast<IterState*>(sums + 3 * nrhs);
+    const double *hr = h->host_report.data(), *hd1 = hr + nrhs, *hd2 = hd1 + nrhs;
     dot_per_rhs(s, q, q, len, nrhs, h->partial, sc);
-    RTE_CUDA_TRY(cudaMemcpyAsync(h->host_sums, sc, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
+    RTE_CUDA_TRY(cudaMemcpyAsync(hq.data(), sc, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
     RTE_CUDA_TRY(cudaStreamSynchronize(s));
-    std::copy(h->host_sums, h->host_sums + nrhs, hq.begin());
     int it = 0, rc = RTE_OK;
     double worst = 0.0, energy = 0.0;
     for (it = 0;; ++it) {
@@ -2425,24 +2429,17 @@ int rte_solve(rte_handle* h, const double* q, double* u, int nrhs, double tol,
         // ||r||^2 and ||u_n - u_{n-1}||^2_{E-K} = delta^T (r_n - r_{n-1})
         {
             Scope scp(h, "axpy");
-            residual_sums(s, r, it > 0 ? delta : nullptr, rprev, len, nrhs, h->partial, sc);
+            residual_sums(s, r, it > 0 ? delta : nullptr, rprev, len, nrhs, h->partial, sums, src, state);
         }
         // the iteration's one synchronisation: its sums, and whether the
         // solves queued since the last one gave up
-        RTE_CUDA_TRY(cudaMemcpyAsync(h->host_sums, sc, sizeof(double) * nrhs * (it > 0 ? 3 : 1),
+        IterState st;
+        RTE_CUDA_TRY(cudaMemcpyAsync(h->host_report.data(), sums, 3 * sizeof(double) * nrhs + sizeof(st),
                                      cudaMemcpyDeviceToHost, s));
-        if (it > 0 && p2)
-            RTE_CUDA_TRY(cudaMemcpyAsync(h->host_status, h->status, sizeof(SolveStatus),
-                                         cudaMemcpyDeviceToHost, s));
-        RTE_TRY(flags_fetch(h));
         RTE_CUDA_TRY(cudaStreamSynchronize(s));
+        std::memcpy(&st, hd2 + nrhs, sizeof(st));
         settle_mk(h);
-        RTE_TRY(flags_check(h));
-        if (it > 0 && p2) {
-            if (h->host_status->timed_out) return fail(RTE_ERR_TIMEOUT, "a bounded grid barrier timed out");
-            h->co_iters = h->host_status->iterations;
-        }
-        const double *hr = h->host_sums, *hd1 = hr + nrhs, *hd2 = hd1 + nrhs;
+        RTE_TRY(state_check(h, st, it > 0 && p2));
         worst = 0.0;
         energy = 0.0;
         bool nan = false;
@@ -2639,7 +2636,6 @@ void rte_destroy(rte_handle* h) {
     for (auto& kv : h->mk_graph) cudaGraphExecDestroy(kv.second);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     if (h->mk_state_host) cudaFreeHost(h->mk_state_host);
-    if (h->host_sums) cudaFreeHost(h->host_sums);
     for (void* p : h->allocs) cudaFreeAsync(p, h->stream);
     cudaStreamSynchronize(h->stream);
     // rte_destroy reports nothing: leave no error behind for the thread's

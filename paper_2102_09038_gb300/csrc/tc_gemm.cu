@@ -279,9 +279,8 @@ int tc_set_wait_cycles(long long cycles) {
     return RTE_OK;
 }
 
-int tc_gemm_error_fetch(cudaStream_t s, int* host) {
-    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(host, g_tc_error, sizeof(int), 0,
-                                           cudaMemcpyDeviceToHost, s));
+int tc_gemm_flag(const int** flag) {
+    RTE_CUDA_TRY(cudaGetSymbolAddress((void**)flag, g_tc_error));
     return RTE_OK;
 }
 
@@ -294,7 +293,8 @@ int tc_gemm_error_check(cudaStream_t s, int flag) {
 
 int tc_gemm_error(cudaStream_t s) {
     int e = 0;
-    RTE_TRY(tc_gemm_error_fetch(s, &e));
+    RTE_CUDA_TRY(cudaMemcpyFromSymbolAsync(&e, g_tc_error, sizeof(int), 0,
+                                           cudaMemcpyDeviceToHost, s));
     RTE_CUDA_TRY(cudaStreamSynchronize(s));
     return tc_gemm_error_check(s, e);
 }

@@ -24,9 +24,9 @@ struct TcGemmArgs {
 int tc_gemm(cudaStream_t s, const TcGemmArgs& g);
 // Reads and clears the device-side timeout flag of the GEMM pipelines.
 int tc_gemm_error(cudaStream_t s);
-// The same in two halves around a synchronisation of the caller's: the copy
-// of the flag to (pinned) host memory, and its check (and clearing) afterwards.
-int tc_gemm_error_fetch(cudaStream_t s, int* host);
+// The flag's address on the current device, and the check (and clearing) of a
+// copy the caller has read.
+int tc_gemm_flag(const int** flag);
 int tc_gemm_error_check(cudaStream_t s, int flag);
 // One wait that runs out, for tests: sets the flag and synchronises s.
 int tc_wait_selftest(cudaStream_t s);
