@@ -160,8 +160,9 @@ typedef struct {
     int mg_sweeps;          /* smoothing sweeps before and after each coarse
                                correction in the multigrid preconditioners   */
     int autotune;           /* 1: time the launch shapes of the SpMM kernels
-                               and tensor-core GEMMs at setup (cached per
-                               shape for the process); 0: fixed shapes       */
+                               and tensor-core GEMMs that the handle's routes
+                               launch at setup (cached per shape for the
+                               process); 0: fixed shapes                     */
     int p1_route;           /* RTE_P1_AUTO (default) | RTE_P1_RICHARDSON |
                                RTE_P1_PCG                                    */
     int e0_route;           /* RTE_E0_AUTO (default) | RTE_E0_DIRECT |

@@ -35,8 +35,9 @@ struct DevLow {
 // Raw device pointers of an assembled system (owned by rte_handle).
 struct DevSystem {
     int m;                     // mesh: m x m squares
-    int tpb_A = 256;           // threads per block of the transport apply (autotuned)
-    int tpb_even = 256;        // threads per block of the even gather (autotuned)
+    // threads per block (autotuned): the transport apply and the even gather of
+    // the handle's FP64 route, and the mixed modes' inner ones
+    int tpb_A = 256, tpb_even = 256, tpb_A_lo = 256, tpb_even_lo = 256;
     int nRp, nRm, nSp, nSm, dP, dM, nnz;
     const double* ell4;        // M_t^+, M_s^+, B_x, B_y in ELL form [4][7][nRp]
     double g, c, gamma;

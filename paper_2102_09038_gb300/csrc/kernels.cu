@@ -553,6 +553,7 @@ __global__ void k_apply_even_s(int m, int nSp, int nrhs, int flags,
 //
 // W consecutive directions per thread: 2 where the pointers are aligned for it,
 // else 1.
+constexpr int kMaxSpmm = 512;   // threads a block, at most (autotuned: 128, 256, 512)
 template <typename T, int N>
 struct alignas(sizeof(T) * N) Pack {
     T v[N];
@@ -562,7 +563,7 @@ struct alignas(sizeof(T) * N) Pack {
 // the "/"-mesh each hat function of a cell has a derivative along x or along y
 // only, but for one: the terms that are zero are left out.
 template <int W>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kMaxSpmm)
 k_grad(int m, int nSp, int nrhs, double sign, const double* __restrict__ cell_D,
        const double* __restrict__ U, double* __restrict__ G) {
     const unsigned nk = (unsigned)nSp / W, total = (unsigned)nrhs * m * m * nk;
@@ -596,7 +597,7 @@ k_grad(int m, int nSp, int nrhs, double sign, const double* __restrict__ cell_D,
 // pointer is set), G as k_grad lays it out.  The stencil sums come before the
 // direction's factors, and the boundary terms on boundary nodes alone.
 template <int W>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kMaxSpmm)
 k_even_grad(int m, int nSp, int nrhs, const double* __restrict__ cell_D, const double* __restrict__ ell4,
             const double* __restrict__ mk, const double* __restrict__ omx, const double* __restrict__ omy,
             const double* __restrict__ G, const double* __restrict__ X, const double* __restrict__ V,
@@ -704,7 +705,7 @@ k_even_grad(int m, int nSp, int nrhs, const double* __restrict__ cell_D, const d
 // zero.  Measured on 128 x 128 / 256 directions: A u 56 us before, 19 now, the gather 94
 // before, 50 now.
 template <typename TOut>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kMaxSpmm)
 k_odd_lo(int m, int nSp, int nrhs, const float* __restrict__ cell_D, const float* __restrict__ A1,
          const float* __restrict__ A2, const float* __restrict__ U, TOut* __restrict__ Z) {
     const unsigned nk = (unsigned)nSp / 4, total = (unsigned)nrhs * m * m * nk;
@@ -749,7 +750,7 @@ k_odd_lo(int m, int nSp, int nrhs, const float* __restrict__ cell_D, const float
     }
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kMaxSpmm)
 k_even_lo(int m, int nSp, int nrhs, const float* __restrict__ cell_D, const float* __restrict__ A1,
           const float* __restrict__ A2, const float* __restrict__ ell4,
           const float* __restrict__ mk, const float* __restrict__ omx,
@@ -1030,43 +1031,43 @@ void apply_grad(cudaStream_t s, const DevSystem& d, const double* U, double* G, 
     // G is the library's own work array: aligned for four values
     const bool two = paired<double>(U);
     const size_t total = (size_t)nrhs * d.m * d.m * (d.nSp / (two ? 2 : 1));
-    const unsigned blocks = (unsigned)((total + 255) / 256);
+    const unsigned blocks = (unsigned)((total + d.tpb_A - 1) / d.tpb_A);
     count_launches(1);
-    if (two) k_grad<2><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, sign, d.cell_D, U, G);
-    else k_grad<1><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, sign, d.cell_D, U, G);
+    if (two) k_grad<2><<<blocks, d.tpb_A, 0, s>>>(d.m, d.nSp, nrhs, sign, d.cell_D, U, G);
+    else k_grad<1><<<blocks, d.tpb_A, 0, s>>>(d.m, d.nSp, nrhs, sign, d.cell_D, U, G);
 }
 
 void apply_even_grad(cudaStream_t s, const DevSystem& d, const double* G, const double* X,
                      const double* V, const double* Q, double* Y, int nrhs) {
     const bool two = paired<double>(X, V, Q, Y);
     const size_t total = (size_t)nrhs * d.nRp * (d.nSp / (two ? 2 : 1));
-    const unsigned blocks = (unsigned)((total + 255) / 256);
+    const unsigned blocks = (unsigned)((total + d.tpb_even - 1) / d.tpb_even);
     count_launches(1);
-    if (two)
-        k_even_grad<2><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.cell_D, d.ell4, d.ang_m, d.ang_omx,
-                                              d.ang_omy, G, X, V, Q, Y);
-    else
-        k_even_grad<1><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.cell_D, d.ell4, d.ang_m, d.ang_omx,
-                                              d.ang_omy, G, X, V, Q, Y);
+    auto run = [&](auto kern) {
+        kern<<<blocks, d.tpb_even, 0, s>>>(d.m, d.nSp, nrhs, d.cell_D, d.ell4, d.ang_m, d.ang_omx,
+                                           d.ang_omy, G, X, V, Q, Y);
+    };
+    if (two) run(k_even_grad<2>);
+    else run(k_even_grad<1>);
 }
 
 void apply_A_lo(cudaStream_t s, const DevSystem& d, const float* U, void* Z, bool bf16, int nrhs) {
     const size_t total = (size_t)nrhs * d.m * d.m * (d.nSp / 4);
-    const unsigned blocks = (unsigned)((total + 255) / 256);
+    const unsigned blocks = (unsigned)((total + d.tpb_A_lo - 1) / d.tpb_A_lo);
     count_launches(1);
     if (bf16)
-        k_odd_lo<__nv_bfloat16><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U,
-                                                       static_cast<__nv_bfloat16*>(Z));
+        k_odd_lo<__nv_bfloat16><<<blocks, d.tpb_A_lo, 0, s>>>(
+            d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U, static_cast<__nv_bfloat16*>(Z));
     else
-        k_odd_lo<float><<<blocks, 256, 0, s>>>(d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U,
-                                               static_cast<float*>(Z));
+        k_odd_lo<float><<<blocks, d.tpb_A_lo, 0, s>>>(
+            d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, U, static_cast<float*>(Z));
 }
 
 void apply_even_lo(cudaStream_t s, const DevSystem& d, const float* Zp, const float* X,
                    const float* V, float* Y, int nrhs) {
     const size_t total = (size_t)nrhs * d.nRp * (d.nSp / 4);
     count_launches(1);
-    k_even_lo<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
+    k_even_lo<<<(unsigned)((total + d.tpb_even_lo - 1) / d.tpb_even_lo), d.tpb_even_lo, 0, s>>>(
         d.m, d.nSp, nrhs, d.lo.cell_D, d.lo.A1, d.lo.A2, d.lo.ell4, d.lo.m, d.lo.omx, d.lo.omy, Zp,
         X, V, Y);
 }

@@ -787,8 +787,9 @@ int setup_multigrid(rte_handle* h, const HostSystem& hs, SetupClock* clk) {
 
 // ------------------------------------------------------------ autotuning
 // Launch shapes chosen by measurement (tune.cpp) on this handle's workspace
-// at max_rhs: the block size of the two SpMM kernels and, in the mixed
-// modes, the tile width of each tensor-core contraction.  Results are
+// at max_rhs: the block sizes of the transport apply and the even gather that
+// the handle's routes launch (FP64, and in the mixed modes the inner ones) and,
+// in the mixed modes, the tile width of each tensor-core contraction.  Results are
 // cached per shape for the process.
 int tune_launches(rte_handle* h) {
     if (!h->opt.autotune) return RTE_OK;
@@ -804,28 +805,40 @@ int tune_launches(rte_handle* h) {
         const size_t lo = d.lo.bf16 ? 2 : 4;
         RTE_CUDA_TRY(cudaMemsetAsync(h->zl1, 0, no * lo, s));
         RTE_CUDA_TRY(cudaMemsetAsync(h->zl2, 0, no * lo, s));
+        RTE_CUDA_TRY(cudaMemsetAsync(h->zf, 0, no * sizeof(float), s));
         RTE_CUDA_TRY(cudaMemsetAsync(h->f1, 0, ne * sizeof(float), s));
         RTE_CUDA_TRY(cudaMemsetAsync(h->xl, 0, ne * lo, s));
     }
-    const int tpb[3] = {128, 256, 512};
     char key[200];
     int b = 1;
-    std::snprintf(key, sizeof key, "apply_A m=%d nS=%d rhs=%d", d.m, d.nSp, nr);
-    RTE_TRY(autotune(s, key, 3, [&](int c) {
-        d.tpb_A = tpb[c];
-        apply_A(s, d, h->e1, h->z1, nr);
-        return ok();
-    }, &b, 1));
-    d.tpb_A = tpb[b];
-    std::snprintf(key, sizeof key, "apply_even m=%d nS=%d rhs=%d", d.m, d.nSp, nr);
-    RTE_TRY(autotune(s, key, 3, [&](int c) {
-        d.tpb_even = tpb[c];
-        apply_even(s, d, h->z2, h->e1, nullptr, h->e2, nr, 3);
-        return ok();
-    }, &b, 1));
-    d.tpb_even = tpb[b];
+    // block size of one of the SpMM kernels; the key names the kernel that the
+    // handle's routes launch
+    auto block_size = [&](const char* name, int& tpb, auto&& launch) -> int {
+        constexpr int sizes[3] = {128, 256, 512};
+        std::snprintf(key, sizeof key, "%s m=%d nS=%d rhs=%d", name, d.m, d.nSp, nr);
+        RTE_TRY(autotune(s, key, 3, [&](int c) {
+            tpb = sizes[c];
+            launch();
+            return ok();
+        }, &b, 1));
+        tpb = sizes[b];
+        return RTE_OK;
+    };
+    if (h->opt.mk_route != RTE_MK_PCG) {
+        RTE_TRY(block_size("apply_A grad", d.tpb_A, [&] { apply_grad(s, d, h->e1, h->z1, nr); }));
+        RTE_TRY(block_size("apply_even grad", d.tpb_even,
+                           [&] { apply_even_grad(s, d, h->z2, h->e1, nullptr, nullptr, h->e2, nr); }));
+    } else {
+        RTE_TRY(block_size("apply_A", d.tpb_A, [&] { apply_A(s, d, h->e1, h->z1, nr); }));
+        RTE_TRY(block_size("apply_even", d.tpb_even,
+                           [&] { apply_even(s, d, h->z2, h->e1, nullptr, h->e2, nr, 3); }));
+    }
     if (!h->mixed) return RTE_OK;
     const bool bf = d.lo.bf16;
+    RTE_TRY(block_size(bf ? "apply_A bf16" : "apply_A fp32", d.tpb_A_lo,
+                       [&] { apply_A_lo(s, d, h->f1, h->zl1, bf, nr); }));
+    RTE_TRY(block_size("apply_even fp32", d.tpb_even_lo,
+                       [&] { apply_even_lo(s, d, h->zf, h->f1, nullptr, h->f2, nr); }));
     const int bns[2] = {128, 256};
     TcGemmArgs g{};
     g.tf32 = !bf;
