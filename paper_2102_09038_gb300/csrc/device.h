@@ -288,11 +288,11 @@ int coarse_cg(cudaStream_t s, const DevSystem& d, const double* B, double* X,
               SolveStatus* status_dev, bool f32_products = false);
 size_t coarse_cg_work_bytes(const DevSystem& d, int nrhs);
 
-// The same on the multigrid route's Kronecker form (ec_kron.cu): whether a
-// system of nRp nodes, d^+ = d and Q terms has it (decided at set-up, with a
-// dense coarsest level), and the solve (work as coarse_cg; limit_ns, trace,
-// cap: the barrier's wait limit and the phase trace of the next launch).
-bool ec_kron_fits(int nRp, int d, int Q, int nrhs);
+// The same on the multigrid route's Kronecker form (ec_kron.cu): whether the
+// handle has it with d^+ <= 16 and a dense coarsest level, and the solve
+// (work as coarse_cg; limit_ns, trace, cap: the barrier's wait limit and the
+// phase trace of the next launch).
+bool ec_kron_takes(const DevSystem& d, int nrhs);
 int ec_kron_cg(cudaStream_t s, const DevSystem& d, const double* B, double* X, int nrhs,
                double tol, int maxit, void* work, SolveStatus* status_dev, bool f32_products,
                unsigned long long limit_ns, unsigned long long* trace, int cap);

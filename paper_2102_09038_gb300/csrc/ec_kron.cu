@@ -797,11 +797,13 @@ int launch_classes(cudaStream_t s, const KronArgs& a) {
 
 }  // namespace
 
-bool ec_kron_fits(int nRp, int d, int Q, int nrhs) {
-    return (Q == 8 || Q == 12 || Q == 16) && (d == 1 || d == 6 || d == 15) &&
-           // 32-bit offsets into the vectors, the diagonal blocks and the
-           // stencils' 16-byte words
-           (double)nrhs * nRp * d < 4e9 && (double)nRp * d * d < 4e9 && 7.0 * (Q / 4) * nRp < 4e9;
+bool ec_kron_takes(const DevSystem& d, int nrhs) {
+    const MGDevice& g = d.ecmg;
+    const bool direct = d.eclu32 != nullptr || d.eclu64 != nullptr;
+    return !direct && (g.Q == 8 || g.Q == 12 || g.Q == 16) && g.dense && g.L >= 1 && g.lev[0].n == d.nRp &&
+           (d.dP == 1 || d.dP == 6 || d.dP == 15) &&
+           // 32-bit offsets into the vectors, the blocks and the stencils
+           (double)nrhs * d.nRp * d.dP < 1e9 && 225.0 * d.nRp < 2e9;
 }
 
 int ec_kron_cg(cudaStream_t s, const DevSystem& d, const double* B, double* X, int nrhs,

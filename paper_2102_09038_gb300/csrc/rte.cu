@@ -731,34 +731,30 @@ int setup_multigrid(rte_handle* h, const HostSystem& hs, SetupClock* clk) {
     } else if (d.dP > 0) {
         MGHost mh;
         const int dP = d.dP;
-        // Kronecker form: Galerkin products of Q scalar stencils
-        const int Q = h->ec_Q;
-        bool kron = ec_kron_fits(hs.nRp, dP, Q, cap);
-        if (kron) {
+        if (h->ec_Q > 0) {   // Kronecker form: Galerkin products of Q scalar stencils
+            const int Q = h->ec_Q;
             RTE_TRY(build_hierarchy(hs.m, hs.st, h->h_ecS, Q, 1, kDenseCoarseNodes, mh));
-            kron = mh.dense_coarse;
-        }
-        if (kron) {
             RTE_TRY(upload_mg_kron(h, mh, cap, dP, Q, h->h_ecG, d.ecmg));
-            const MGHostLevel& L = mh.levels.back();
-            const int n = (L.m + 1) * (L.m + 1), N = n * dP;
-            const size_t nnz = L.st.col.size(), dd = (size_t)dP * dP;
-            std::vector<double> A((size_t)N * N, 0.0);
-            for (int i = 0; i < n; ++i)
-                for (int k = L.st.ptr[i]; k < L.st.ptr[i + 1]; ++k) {
-                    const int j = L.st.col[k];
-                    for (int q = 0; q < Q; ++q) {
-                        const double sq = L.vals[(size_t)q * nnz + k];
-                        if (sq == 0.0) continue;
-                        const double* g = &h->h_ecG[(size_t)q * dd];
-                        for (int a = 0; a < dP; ++a)
-                            for (int b = 0; b < dP; ++b)
-                                A[(size_t)(i * dP + a) * N + j * dP + b] += sq * g[a * dP + b];
+            if (d.ecmg.dense) {
+                const MGHostLevel& L = mh.levels.back();
+                const int n = (L.m + 1) * (L.m + 1), N = n * dP;
+                const size_t nnz = L.st.col.size(), dd = (size_t)dP * dP;
+                std::vector<double> A((size_t)N * N, 0.0);
+                for (int i = 0; i < n; ++i)
+                    for (int k = L.st.ptr[i]; k < L.st.ptr[i + 1]; ++k) {
+                        const int j = L.st.col[k];
+                        for (int q = 0; q < Q; ++q) {
+                            const double sq = L.vals[(size_t)q * nnz + k];
+                            if (sq == 0.0) continue;
+                            const double* g = &h->h_ecG[(size_t)q * dd];
+                            for (int a = 0; a < dP; ++a)
+                                for (int b = 0; b < dP; ++b)
+                                    A[(size_t)(i * dP + a) * N + j * dP + b] += sq * g[a * dP + b];
+                        }
                     }
-                }
-            RTE_TRY(upload_coarse_inverse(h, N, A, d.ecmg));
+                RTE_TRY(upload_coarse_inverse(h, N, A, d.ecmg));
+            }
         } else {
-            mh = MGHost();
             RTE_TRY(build_hierarchy(hs.m, hs.st, h->h_ec, 1, dP, kDenseCoarseNodes, mh));
             RTE_TRY(upload_mg(h, mh, cap, dP, true, d.ecmg));
             if (d.ecmg.dense) {
