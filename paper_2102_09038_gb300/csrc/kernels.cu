@@ -1277,8 +1277,8 @@ void fill_uniform(cudaStream_t s, double* x, size_t n, unsigned long long seed) 
 // k with 16 partial sums each, reduced across the warp by halving exchanges
 // (31 shuffles leave lane j holding the sum of column j mod 16).
 // SUB: of x - sub instead.  (The variants of these two kernels are compiled
-// apart: with the choice made at run time the plain ones ran 1.0 to 1.15 and
-// 1.05 to 1.9 times as long.)
+// apart, and their loops written apart below: with the choice made at run time
+// the plain ones ran 1.0 to 1.15 and 1.05 to 1.9 times as long.)
 template <typename T, bool SUB>
 __global__ void __launch_bounds__(256) k_restrict(int rows, int nSp, int dP, const double* __restrict__ x,
                                                   const float* __restrict__ sub,
@@ -1328,17 +1328,28 @@ __global__ void __launch_bounds__(256) k_prolong(int rows, int nSp, int dP, cons
 #pragma unroll
     for (int j = 0; j < 16; ++j) u[j] = __shfl_sync(0xffffffffu, mine, j);
     double* xr = x + (size_t)row * nSp;
-    for (int k = lane; k < nSp; k += 32) {
+    auto value = [&](int k) {
         T acc = T(0);
 #pragma unroll
         for (int j = 0; j < 16; ++j)
             if (j < dP) acc = fma(u[j], __ldg(WT + (size_t)j * nSp + k), acc);
-        const double v = beta == 0.0 ? (double)acc : beta * xr[k] + (double)acc;
-        if constexpr (UPDATE) {
-            U[(size_t)row * nSp + k] -= v;
-            D[(size_t)row * nSp + k] = -v;
-        } else {
-            xr[k] = v;
+        return (double)acc;
+    };
+    if constexpr (UPDATE) {
+        // four trips' loads at once in FP32 (96 x 96 / 2048 triangles: 92 us,
+        // 168 one by one); in FP64 that takes 88 registers and is slower (64 x
+        // 64 / 512: 61 us against 47)
+        double *Ur = U + (size_t)row * nSp, *Dr = D + (size_t)row * nSp;
+#pragma unroll (sizeof(T) == 4 ? 4 : 1)
+        for (int k = lane; k < nSp; k += 32) {
+            const double x0 = beta == 0.0 ? 0.0 : xr[k], u0 = Ur[k], v = beta * x0 + value(k);
+            Ur[k] = u0 - v;
+            Dr[k] = -v;
+        }
+    } else {
+        for (int k = lane; k < nSp; k += 32) {
+            const double v = value(k);
+            xr[k] = beta == 0.0 ? v : beta * xr[k] + v;
         }
     }
 }
