@@ -187,32 +187,6 @@ def fp64_peak_tflops(torch):
     return 2.0 * n ** 3 / best / 1e12
 
 
-# DRAM traffic of a timing scope's kernel from an ncu launch list of this
-# benchmark's own workload (`bench.py --profile-once`; the summary and the
-# command are in profiles/launches_checkerboard_128x128_T512_mixed_bf16.md):
-# dram__bytes_read.sum + dram__bytes_write.sum averaged over the kernel's
-# launches in one solve, the source file the kernel lives in and that file's
-# SHA-256 prefix at the capture.  The bench reports it only for the workload
-# it was captured on, and null once the source has changed since.
-PROFILED_DRAM = {
-    'coarse_cg': dict(source='paper_2102_09038_gb300/csrc/mg.cu', sha='e29a65ac179f3b0b',
-                      workload='checkerboard_128x128_T512_g0.90_c0.99',
-                      bytes_per_launch=1.829e9, coarse_iters=5,
-                      note='ncu launch list, 16 launches of k_ec_pcg<0> in one solve '
-                           '(5 CG iterations each)'),
-    'e0_direct': dict(source='paper_2102_09038_gb300/csrc/e0_direct.cu', sha='170f9aa09a001022',
-                      workload='checkerboard_128x128_T512_g0.90_c0.99',
-                      bytes_per_launch=4.736e9,
-                      note='ncu launch list, 32 launches of k_e0_direct_tma in one solve'),
-}
-
-
-def source_sha(rel):
-    import hashlib
-    with open(os.path.join(ROOT, rel), 'rb') as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
-
-
 def e0_units(d, nrhs, info):
     """Work units of one E_0^{-1} launch: (node, column) items times the
     launch's CG iterations, each weighted by the fraction of direction quads
@@ -293,8 +267,9 @@ def roofline_of(name, total_ms, launches, d, nrhs, info, peaks, src, fp64_peak, 
     (kernel_work) over the scope's mean launch time, against the measured
     peak of its bound; fp64_peak() gives the measured FP64 rate (timed only
     when a scope needs it).  The algorithmic counts are of the method's dense
-    steps; where the library does
-    less, performed_work says how much (performed, performed_frac)."""
+    steps; where the library does less, performed_work says how much
+    (performed, performed_frac), and that is what the line reports as frac
+    (reported)."""
     avg_ms = total_ms / max(launches, 1)
     roof = dict(kernel=name, bound=None, achieved=None, peak=None, unit=None, frac=None,
                 launches=launches, avg_ms=avg_ms)
@@ -325,6 +300,18 @@ def roofline_of(name, total_ms, launches, d, nrhs, info, peaks, src, fp64_peak, 
     if done is not None:
         roof.update(performed=done, performed_frac=roof['frac'] * done / amount)
     return roof
+
+
+def reported(roof):
+    """A scope's roofline as the line prints it: where the library does less
+    than the dense count, achieved and frac are of the work performed, the
+    dense ones stand beside them, and the dense design's bytes are left out."""
+    if roof.get('performed_frac') is None:
+        return roof
+    out = {k: v for k, v in roof.items() if k not in ('impl_bytes', 'impl_frac', 'performed_frac')}
+    out.update(frac=roof['performed_frac'], dense_frac=roof['frac'],
+               achieved=roof['achieved'] * roof['performed_frac'] / roof['frac'])
+    return out
 
 
 def performed_work(name, d, nrhs, tol):
@@ -370,12 +357,13 @@ def scope_rooflines(tim, d, nrhs, info, peaks, src, fp64_peak, tol, count=4):
 
 def kernel_impl_bytes(name, d, nrhs, info):
     """The bytes of the E_0 kernels' own design, per launch (kept beside the
-    algorithmic count; the direct route's are those of dense padded rows,
-    performed_work has what its packed records move): per V-cycle and active (node, column) the
-    12 CG-vector passes of the precision w and the iterate read and written,
+    algorithmic count).  Multigrid route: per V-cycle and active (node, column)
+    the 12 CG-vector passes of the precision w and the iterate read and written,
     the V-cycle's 17 FP32 array passes per level (4^-l of the level-0 size)
     and the coarsest level's dense per-direction inverses, plus the FP64
-    right-hand side and solution once."""
+    right-hand side and solution once.  Direct route: dense rows padded to 16
+    bytes with four coupling coefficients per item (performed_work has what the
+    packed records move, which is what the line reports)."""
     nRp, nS = d['nRp'], d['nSp']
     if name in ('e0_direct', 'e0_direct64'):
         # the factor rows padded to ld (a multiple of 4), read twice per
@@ -480,19 +468,6 @@ def run_ours(args):
     d['e0_levels'] = levels_of(args.mesh)
     d['mesh'] = args.mesh
     d['dP'] = solver.d_plus
-    traffic, traffic_note = None, 'no ncu capture of the current kernel source'
-    prof = PROFILED_DRAM.get(top[0])
-    if prof:
-        if source_sha(prof['source']) != prof['sha']:
-            traffic_note = 'kernel changed since its ncu capture'
-        elif (prof['workload'] != WORKLOAD['workload'] or args.mesh != WORKLOAD['mesh']
-              or 8 * 4 ** args.levels != WORKLOAD['sphere_triangles']):
-            traffic_note = 'ncu capture taken on another workload'
-        elif prof.get('coarse_iters') not in (None, last_info.get('coarse_iters')):
-            traffic_note = 'ncu capture taken at another coarse iteration count'
-        else:
-            traffic = prof['bytes_per_launch']
-            traffic_note = prof['note']
     fp64_rate = []
 
     def fp64_peak():
@@ -501,7 +476,8 @@ def run_ours(args):
         return fp64_rate[0]
 
     roof, rooflines = scope_rooflines(tim, d, p.nrhs, last_info, peaks, src, fp64_peak, p.tol)
-    roof.update(traffic=traffic, traffic_source=traffic_note)
+    roof, rooflines = reported(roof), [reported(r) for r in rooflines]
+    roof.update(traffic=None, traffic_source='not captured at this size (profiles/ has 64 x 64)')
     share = {k: round(v[0] / sum(x[0] for x in tim.values()), 4)
              for k, v in tim.items()}
 
