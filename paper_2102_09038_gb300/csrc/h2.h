@@ -74,8 +74,12 @@ void h2_lists(const H2Plan& P, const H2Pool& pool, H2Lists& L);
 // when an output has no entries.
 H2List h2_group_list(const H2List& l, int G);
 // Whether a list's groups save enough: the tiles read by groups (a 16 KB input
-// and its 8 KB matrices) against singly, where blocks have entries enough to
-// hide their ends.
+// and its 8 KB matrices) at most 0.8 of those read singly, in blocks of 8
+// entries or more.  Both sides, us an apply with no list in pairs, with these,
+// with every list: S^+ of 16384 directions, 2048 rows 1209, 1065, 1038; S^- of
+// 4096, 2500 rows 860, 784, 771; S^+ of 4096 (couplings at 0.81: singly), 8000
+// rows 969, 955, 897; S^+ of 256 (4 entries: singly), 39000 rows 181, 178, 160.
+// The line is on the safe side: short lists gain from pairs too.
 bool h2_group_pays(const H2List& l, const H2List& grouped);
 // Whether a call takes the groups: every SM gets two blocks twice over.
 inline bool h2_takes_groups(int groups, int row_tiles, int sms) {

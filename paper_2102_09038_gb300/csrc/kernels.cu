@@ -1085,8 +1085,13 @@ int device_sm_count() {
 
 template <int EPI, typename... Args>
 static int gemm_f64_epi(cudaStream_t s, int M, int N, Args... args) {
-    // products on the busiest SM, per step of K; a little more for the
-    // operand traffic of each smaller tile
+    // Products on the busiest SM, per step of K, and 8 % more for the operand
+    // traffic of each smaller tile, so that calls with many tiles stay at 64 x
+    // 64.  Both sides (us, 64 x 64, 32 x 64, 32 x 32, 16 x 32; taken: *):
+    // 324 x 192 x 128 147, 77, 43, 26*; 512 x 192 x 128 147, 77, 43*, 41;
+    // 2048 x 192 x 128 148, 145, 111*, 111; 6400 x 192 x 128 284*, 284, 284, 286;
+    // 1152 x 512 x 768 789*, 773, 773, 778; 8192 x 768 x 512 5728*, 5462, 5349,
+    // 5305 (the 8 % could be less: the operands come from L2 in time).
     const int tiles[4][2] = {{64, 64}, {32, 64}, {32, 32}, {16, 32}};
     const double sms = device_sm_count();
     int best = 0;

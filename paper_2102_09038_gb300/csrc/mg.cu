@@ -1087,7 +1087,11 @@ __device__ __forceinline__ float ec_apply(const MGDeviceLevel& L, const float* x
 // t_q = sum_dir S_q(i, nbr) x_nbr (lane a holds component a), then
 // y_a = sum_q sum_b G_q[a][b] t_q[b] with t_q[b] from lane b of the group.
 // The stencils are node-major [n][7][Qp]; sG holds the G_q in shared memory.
-// Every lane of the warp must call this (shuffles).
+// Every lane of the warp must call this (shuffles).  Systems of 1 to 3 sigma
+// classes take ec_kron.cu instead up to its 32-bit offsets, so this runs only
+// beyond them (meshes above 2980, or 1e9 values of a coarse vector).  Without
+// it the compiler's code for the explicit blocks is slower (48 x 48 in four
+// classes: 364 -> 375 us a solve; d = 28 on 32 x 32: 911 -> 982).
 constexpr int kEcMaxQ = 16;
 __device__ __forceinline__ float ec_apply_kron(const MGDeviceLevel& L, const float* sG, int Q,
                                                const float* x, int r, int i, int d, int G,

@@ -16,9 +16,11 @@
 // tile's epilogue (a division per element, 64 to 128 KB of stores) takes about
 // as long as its MMAs, and one tile per block exposed both.  Measured in a
 // solve, 32768 x 768 x 768 BF16: with the shifted inverse in the epilogue 152
-// -> 79 us, the plain product to FP32 81 -> 57 us.  Every wait on an mbarrier
-// is bounded: on timeout the kernel records an error flag and leaves instead
-// of hanging.
+// -> 79 us, the plain product to FP32 81 -> 57 us.  Calls of at most one tile
+// an SM gain nothing from it and lose nothing (a whole rte_gemm_lowp call, one
+// tile per block of 128 threads before and now: 128 x 256 x 768 BF16 48 and 46
+// us, 1000 x 100 x 128 TF32 47 and 46).  Every wait on an mbarrier is bounded:
+// on timeout the kernel records an error flag and leaves instead of hanging.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -993,7 +995,8 @@ int ozaki_split(cudaStream_t s, const double* X, int rows, int K, int S, void* o
     // 32 rows a block of 256 threads where that gives every SM two blocks,
     // else 16, or 8, rows of 512 or 1024: a short operand is then cut by as
     // many warps as a long one (1500 x 384 x 3072 at seven slices, the whole
-    // product: 279 -> 229 us)
+    // product: 279 -> 229 us).  1500 x 384 in the static scratch, 256, 512 and
+    // 1024 threads: K = 768 93, 86, 86 us; up to K = 512 all within 1 us.
     const int sms = device_sm_count();
     const int R = rows >= 64 * sms ? 32 : rows >= 16 * sms ? 16 : 8;
     const int threads = R == 32 ? 256 : K >= 512 ? 1024 : 512;
