@@ -70,9 +70,10 @@ struct rte_handle {
     float* zf = nullptr;
     double *partial = nullptr, *sc = nullptr;                               // reductions
     // What the outer iteration's one synchronisation brings to the host in one
-    // copy: the sums of ||q||^2 and of the residual [3][cap_rhs], then the
-    // iteration's state.  Pageable on the host: freeing pinned memory waits for
-    // every stream of the device, and rte_destroy waits for the handle's alone.
+    // copy: the residual's sums [3][nrhs], then the iteration's state.  Pageable
+    // on the host: freeing pinned memory waits for every stream of the device,
+    // and rte_destroy is to wait for the handle's alone (it still frees
+    // mk_state_host on Algorithm 1's route).
     char* report = nullptr;
     std::vector<double> host_report;
     void* e0work = nullptr;
